@@ -21,20 +21,26 @@
 // the same rows (the 16x32bx2 TMEM access shape), and combine the row maximum
 // and the row sum with one shuffle.
 //
-// Softmax (lazy rescaling, base 2): each row keeps -m and its row sum l.  A
-// tile's scores are t = s log2(e)/sqrt(d) - m; when the row's largest t of
-// the tile exceeds 2^3 (or on the first tile of the item) m is raised to the
-// tile maximum and the O row and l are scaled by 2^(m_old - m_new) (a warp
-// takes that path when any of its rows needs it; the O row is rescaled after
-// the previous P V has finished and before this tile's P is handed over).
-// p = 2^t enters the row sum in fp32 and the product rounded to bf16.
+// Softmax (lazy rescaling, base 2): two warpgroups take the tiles of an item
+// in turn, so a tile's softmax may last two tile periods.  -m, the running
+// maximum that both use for a row, goes from one to the other through shared
+// memory (sm.m): after its tile's row maximum a warp waits for -m of the tile
+// before, raises m if the tile's largest t = s log2(e)/sqrt(d) - m exceeds 2^3
+// (or on the first tile of the item), and passes it on before it evaluates the
+// exponentials.  A raised m scales the O row by 2^(m_old - m_new), after the
+// previous P V has finished and before this tile's P is handed over (a warp
+// takes that path when any of its rows needs it).  Each group keeps the row
+// sum of its own tiles; the group of the item's last tile adds the other's and
+// writes O.  p = 2^t enters the row sum in fp32 and the product rounded to bf16.
 //
-// Warp roles (256 threads, one persistent CTA per SM):
-//   warps 0-3  softmax + epilogue: warp w owns TMEM lane quarter w
-//   warp  4    TMA producer: Q (per item) and the K pairs
-//   warp  5    TMA producer: the V blocks
-//   warp  6    S = Q K^T issuer and TMEM owner
-//   warp  7    O += P V issuer
+// Warp roles (384 threads, one persistent CTA per SM):
+//   warps 0-3, 4-7  softmax of the even / odd tiles of the CTA + epilogue: warp w owns TMEM lane quarter w mod 4
+//   warp  8    TMA producer: Q (per item) and the K pairs
+//   warp  9    TMA producer: the V blocks
+//   warp 10    S = Q K^T issuer and TMEM owner
+//   warp 11    O += P V issuer
+// (QN = 128: the softmax groups hold 128 scores a thread, so they take 208
+// registers and leave the last warpgroup 88.)
 // Buffers (shared memory): Q (QN = 64: two 16 KB buffers, so the next item's
 // Q arrives during this one; QN = 128: one of 32 KB), K pairs in a 3-deep
 // ring (32 KB each), V blocks in a ring of single 16 KB blocks (6 for QN = 64,
@@ -43,6 +49,20 @@
 // next tile runs while the softmax of this one does.  Every mbarrier wait is
 // bounded; a wait that gives up records ROLA_ERR_TIMEOUT in the status word
 // and the CTA stops issuing, drains what it issued and releases its TMEM.
+//
+// What bounds it, measured at the 720p layer (40 heads, 75600 tokens, 118 of
+// 1182 blocks kept; clock64 around every wait of one CTA):
+//   - a producer warp that predicates each step on lanes spends ~640 cycles a
+//     16 KB block on fixed latencies (mbarrier wait 110-170, expect_tx ~50, a TMA
+//     instruction 80), whatever the ring's depth; one elected thread that keeps
+//     the next block ids in registers needs ~350 for two boxes.  14.76 -> 11.85
+//     ms (QN = 64); the L2 itself delivers a 16 KB block per 248 cycles and SM.
+//   - two softmax groups in turn: 11.85 -> 11.5 ms (QN = 64), 8.2 -> 7.3 ms (QN = 128).
+//   - QN = 64 now takes 1137 cycles a tile: 1024 of tensor work (an M = 64
+//     product runs at half the M = 128 rate) and 144 KB through the shared
+//     memory (1125 at 128 B/cycle).  QN = 128 takes ~1400 cycles against the
+//     same 1024, its softmax groups 2350 of the 2800 cycles they have.  The SM
+//     clock falls to 1.73-1.82 GHz (from 2.07) under the denser kernels.
 //
 // Per 64-query block and 128-key tile the shared memory sees 64 KB of TMA
 // writes (K, V) and 80 KB of operand reads (Q 16, K 32, V 32) for 4.2 MFLOP,
@@ -60,9 +80,9 @@ namespace {
 
 using namespace tc;
 
-constexpr int kSoftmaxWarps = 4;
-constexpr int kProducerKWarp = 4, kProducerVWarp = 5, kMmaWarp = 6, kPvWarp = 7;
-constexpr int kThreads = 256;
+constexpr int kWarpsPerGroup = 4;                    // a softmax warpgroup
+constexpr int kProducerKWarp = 8, kProducerVWarp = 9, kMmaWarp = 10, kPvWarp = 11;
+constexpr int kThreads = 384;
 constexpr uint32_t kKPairBytes = 128 * 128 * 2;      // a pair of key blocks [d-chunk][block][64 rows][64]
 constexpr uint32_t kVBlockBytes = 64 * 128 * 2;      // one key block of v [d-chunk][64 rows][64]
 constexpr uint32_t kTmemCols = 512;
@@ -85,13 +105,15 @@ struct Cfg {
     static constexpr uint32_t kSmemTiles = kSmemV + VB * kVBlockBytes;
     static constexpr int Q_FULL = 0, Q_EMPTY = Q_FULL + QB, K_FULL = Q_EMPTY + QB, K_EMPTY = K_FULL + KS,
                          V_FULL = K_EMPTY + KS, V_EMPTY = V_FULL + VB, S_FULL = V_EMPTY + VB, S_EMPTY = S_FULL + 2,
-                         P_FULL = S_EMPTY + 2, PV_DONE = P_FULL + 2, O_FULL = PV_DONE + 2, O_EMPTY = O_FULL + 1,
-                         DRAIN = O_EMPTY + 1, NUM_BARS = DRAIN + 2;
+                         P_FULL = S_EMPTY + 2, PV_DONE = P_FULL + 2, O_FULL = PV_DONE + 4, O_EMPTY = O_FULL + 2,
+                         M_READY = O_EMPTY + 1, L_READY = M_READY + 8, DRAIN = L_READY + 8, NUM_BARS = DRAIN + 2;
     static_assert(kSmemTiles % 1024 == 0, "the control block follows the 1024-aligned tiles");
 };
 
 template <int QN>
 struct Ctrl {
+    float m[2][QN];                      // -m of every row after an even / odd tile
+    float2 l[2][QN];                     // (row sum, its -m) of the group that does not end item k, by k & 1
     uint64_t bar[Cfg<QN>::NUM_BARS];
     uint32_t tmem_base;
     int abort;
@@ -194,6 +216,12 @@ __device__ __forceinline__ void fadd2(float& a, float& b, float p, float q)
         : "+f"(a), "+f"(b) : "f"(p), "f"(q));
 }
 
+// Moves registers between the warpgroups (executed by all warps of one).
+template <int R>
+__device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(R)); }
+template <int R>
+__device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(R)); }
+
 template <int QN>
 __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                                                                        const __grid_constant__ CUtensorMap map_k,
@@ -206,7 +234,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
     constexpr int Q_FULL = C::Q_FULL, Q_EMPTY = C::Q_EMPTY, K_FULL = C::K_FULL, K_EMPTY = C::K_EMPTY,
                   V_FULL = C::V_FULL, V_EMPTY = C::V_EMPTY, S_FULL = C::S_FULL, S_EMPTY = C::S_EMPTY,
                   P_FULL = C::P_FULL, PV_DONE = C::PV_DONE, O_FULL = C::O_FULL, O_EMPTY = C::O_EMPTY,
-                  DRAIN = C::DRAIN;
+                  M_READY = C::M_READY, L_READY = C::L_READY, DRAIN = C::DRAIN;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     // the 128-byte-swizzle atoms need a 1024-byte aligned base; the kernel has
     // no static shared memory, so the dynamic block starts on the window base
@@ -239,20 +267,24 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar(S_FULL + i), 1);
-            mbar_init(bar(S_EMPTY + i), kSoftmaxWarps);
-            mbar_init(bar(P_FULL + i), kSoftmaxWarps);
-            mbar_init(bar(PV_DONE + i), 1);
+            mbar_init(bar(S_EMPTY + i), kWarpsPerGroup);
+            mbar_init(bar(P_FULL + i), kWarpsPerGroup);
+            mbar_init(bar(O_FULL + i), 1);
             mbar_init(bar(DRAIN + i), 1);
         }
-        mbar_init(bar(O_FULL), 1);
-        mbar_init(bar(O_EMPTY), kSoftmaxWarps);
+        for (int i = 0; i < 4; ++i) mbar_init(bar(PV_DONE + i), 1);
+        for (int i = 0; i < 8; ++i) {
+            mbar_init(bar(M_READY + i), 1);
+            mbar_init(bar(L_READY + i), 1);
+        }
+        mbar_init(bar(O_EMPTY), kWarpsPerGroup);
         fence_mbar_init();
     }
     if (warp == kMmaWarp) {
         tmem_alloc(smem_u32(&sm.tmem_base), kTmemCols);
         tmem_relinquish();
     }
-    if ((warp == kProducerKWarp || warp == kProducerVWarp) && lane == 0) {
+    if (warp == kProducerKWarp && lane == 0) {
         tma_prefetch_desc(&map_q);
         tma_prefetch_desc(&map_k);
         tma_prefetch_desc(&map_v);
@@ -263,82 +295,84 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
     const uint32_t tmem = sm.tmem_base;
     volatile int* abort = &sm.abort;
 
+    if constexpr (QN == 128) {
+        if (warp >= kProducerKWarp) regs_dec<88>();    // the softmax groups take 208: 208 + 208 + 88 = 3 x 168
+    }
     if (warp == kProducerKWarp || warp == kProducerVWarp) {
         // ------------------------------------------------------------ TMA producers
-        // K warp: lane 0 loads Q (one box); lanes 2h + c load d-chunk c of
-        // block h of the K pair (8 KB boxes, [chunk][block][row] so that the
-        // pair is one N = 128 operand).  V warp: lanes 2h + c load d-chunk c of
-        // block h into its slot of the ring of single blocks ([chunk][row]).
-        // A lane's copies are processed one after another, so every copy of a
-        // tile gets a lane of its own.
+        // One elected thread per warp.  K warp: Q (one box per item) and the K
+        // pairs, 8 KB boxes in [chunk][block][row] order so that the pair is
+        // one N = 128 operand.  V warp: a 16 KB box ([chunk][row]) per block
+        // into its slot of the ring of single blocks.
         const bool is_v = warp == kProducerVWarp;
-        const int h = lane >> 1;                        // block of the pair
-        const int kc = lane & 1;                        // d-chunk
-        int k = 0, issued_q = 0, issued_k = 0, issued_vb = 0;
-        bool ok = true;
-        for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x, ++k) {
-            const int bh = item / nI, qb = item - bh * nI;
-            const int32_t* kept = p.kv_idx + (size_t)item * s.n_keep;
-            if (!is_v) {
-                const int qs = k % QB;
-                if (k >= QB) ok = mbar_wait(bar(Q_EMPTY + qs), ((k / QB) - 1) & 1, abort, s.wait_limit_ns);
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (!ok) break;
-                if (lane == 0) {
+        if (elect_one()) {
+            int k = 0, g = 0, issued_q = 0, issued = 0;
+            bool ok = true;
+            for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x, ++k) {
+                const int bh = item / nI, qb = item - bh * nI;
+                const int32_t* kept = p.kv_idx + (size_t)item * s.n_keep;
+                int ja_n = __ldg(kept), jb_n = s.n_keep > 1 ? __ldg(kept + 1) : -1;     // block ids, one tile ahead
+                if (!is_v) {
+                    const int qs = k % QB;
+                    if (k >= QB && !(ok = mbar_wait(bar(Q_EMPTY + qs), ((k / QB) - 1) & 1, abort, s.wait_limit_ns)))
+                        break;
                     mbar_expect_tx(bar(Q_FULL + qs), kQBytes);
                     tma_load_4d(sbase + kSmemQ + qs * kQBytes, &map_q, bar(Q_FULL + qs), 0, qb * QN, 0, bh);
+                    ++issued_q;
                 }
-                ++issued_q;
-            }
-            for (int t = 0; t < T; ++t) {
-                const int g = k * T + t;
-                const int ja = __ldg(kept + 2 * t);
-                const int jb = 2 * t + 1 < s.n_keep ? __ldg(kept + 2 * t + 1) : -1;
-                const int nblk = jb >= 0 ? 2 : 1;
-                if (is_v) {
-                    const int c = k * s.n_keep + 2 * t + h;       // cumulative block index of block h
-                    const int slot = c % VB;
-                    bool okl = true;
-                    if (lane < 4 && kc == 0 && h < nblk && c >= VB)
-                        okl = mbar_wait(bar(V_EMPTY + slot), ((c / VB) - 1) & 1, abort, s.wait_limit_ns);
-                    ok = __shfl_sync(0xffffffffu, okl, 0) && __shfl_sync(0xffffffffu, okl, 2);
-                    if (!ok) break;
-                    if (lane < 4 && kc == 0 && h < nblk) mbar_expect_tx(bar(V_FULL + slot), kVBlockBytes);
-                    __syncwarp();
-                    if (lane < 4 && h < nblk)
-                        tma_load_3d(sbase + kSmemV + slot * kVBlockBytes + kc * 8192, &map_v, bar(V_FULL + slot),
-                                    kc * 64, (h ? jb : ja) * 64, bh);
-                    issued_vb += nblk;
-                } else {
-                    const int st = g % KS;
-                    if (g >= KS) ok = mbar_wait(bar(K_EMPTY + st), ((g / KS) - 1) & 1, abort, s.wait_limit_ns);
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
-                    if (!ok) break;
-                    // test hook: the first K copy of the CTA is never issued, so the waits on it run out
-                    const bool skip = (s.debug_flags & ROLA_DEBUG_SKIP_FIRST_K_COPY) && g == 0;
-                    if (lane == 0 && !skip) mbar_expect_tx(bar(K_FULL + st), nblk * 16384u);
-                    __syncwarp();
-                    if (lane < 4 && h < nblk && !skip)
-                        tma_load_3d(sbase + kSmemK + st * kKPairBytes + kc * 16384 + h * 8192, &map_k,
-                                    bar(K_FULL + st), kc * 64, (h ? jb : ja) * 64, bh);
-                    ++issued_k;
+                for (int t = 0; t < T; ++t, ++g) {
+                    const int ra = ja_n * 64, rb = jb_n * 64;
+                    const bool two = jb_n >= 0;                 // the last tile of an odd n_keep holds one block
+                    if (t + 1 < T) {
+                        ja_n = __ldg(kept + 2 * t + 2);
+                        jb_n = 2 * t + 3 < s.n_keep ? __ldg(kept + 2 * t + 3) : -1;
+                    }
+                    if (is_v) {
+                        const int c = k * s.n_keep + 2 * t;     // cumulative block index of the tile's first block
+                        const int sa = c % VB, sb = (c + 1) % VB;
+                        if (c >= VB && !(ok = mbar_wait(bar(V_EMPTY + sa), ((c / VB) - 1) & 1, abort, s.wait_limit_ns)))
+                            break;
+                        mbar_expect_tx(bar(V_FULL + sa), kVBlockBytes);
+                        tma_load_4d(sbase + kSmemV + sa * kVBlockBytes, &map_v, bar(V_FULL + sa), 0, ra, 0, bh);
+                        issued = c + 1;
+                        if (!two) continue;
+                        if (c + 1 >= VB &&
+                            !(ok = mbar_wait(bar(V_EMPTY + sb), (((c + 1) / VB) - 1) & 1, abort, s.wait_limit_ns)))
+                            break;
+                        mbar_expect_tx(bar(V_FULL + sb), kVBlockBytes);
+                        tma_load_4d(sbase + kSmemV + sb * kVBlockBytes, &map_v, bar(V_FULL + sb), 0, rb, 0, bh);
+                        issued = c + 2;
+                    } else {
+                        const int st = g % KS;
+                        if (g >= KS && !(ok = mbar_wait(bar(K_EMPTY + st), ((g / KS) - 1) & 1, abort, s.wait_limit_ns)))
+                            break;
+                        issued = g + 1;
+                        // test hook: the first K copy of the CTA is never issued, so the waits on it run out
+                        if ((s.debug_flags & ROLA_DEBUG_SKIP_FIRST_K_COPY) && g == 0) continue;
+                        const uint32_t dst = sbase + kSmemK + st * kKPairBytes, full = bar(K_FULL + st);
+                        mbar_expect_tx(full, two ? 32768u : 16384u);
+                        tma_load_3d(dst, &map_k, full, 0, ra, bh);
+                        tma_load_3d(dst + 16384, &map_k, full, 64, ra, bh);
+                        if (two) {
+                            tma_load_3d(dst + 8192, &map_k, full, 0, rb, bh);
+                            tma_load_3d(dst + 24576, &map_k, full, 64, rb, bh);
+                        }
+                    }
                 }
             }
-        }
-        if (!ok && lane == 0) record_timeout(p, is_v ? 4 : 1);
-        // every copy this warp issued lands before the CTA exits (bounded by time only)
-        if (lane == 0) {
+            if (!ok) record_timeout(p, is_v ? 4 : 1);
+            // every copy this thread issued lands before the CTA exits (bounded by time only)
             int never = 0;
             for (int u = issued_q > QB ? issued_q - QB : 0; u < issued_q; ++u)
                 mbar_wait(bar(Q_FULL + u % QB), (u / QB) & 1, &never, s.wait_limit_ns);
-            const int NS = is_v ? VB : KS, issued = is_v ? issued_vb : issued_k;
+            const int NS = is_v ? VB : KS;
             const int full0 = is_v ? V_FULL : K_FULL;
             for (int u = issued > NS ? issued - NS : 0; u < issued; ++u)
                 mbar_wait(bar(full0 + u % NS), (u / NS) & 1, &never, s.wait_limit_ns);
         }
     } else if (warp == kMmaWarp || warp == kPvWarp) {
         // ------------------------------------------------------------ MMA issuers
-        if (lane == 0) {
+        if (elect_one()) {
             const bool pv = warp == kPvWarp;
             const uint32_t id_qk = idesc_bf16(QN, 128, false, false);
             const uint32_t id_pv = idesc_bf16(QN, 128, false, true);
@@ -377,12 +411,13 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
                         const bool half = 2 * t + 1 >= s.n_keep;
                         const int c0 = k * s.n_keep + 2 * t;
                         const int va = c0 % VB, vb = (c0 + 1) % VB;
-                        if (!(ok = mbar_wait(bar(P_FULL + pb), (g >> 1) & 1, abort, s.wait_limit_ns))) break;
+                        // (V and O first: they are there long before P, whose wait is on the critical chain)
                         if (!(ok = mbar_wait(bar(V_FULL + va), (c0 / VB) & 1, abort, s.wait_limit_ns))) break;
                         if (!half && !(ok = mbar_wait(bar(V_FULL + vb), ((c0 + 1) / VB) & 1, abort, s.wait_limit_ns)))
                             break;
                         if (t == 0 && k >= 1 && !(ok = mbar_wait(bar(O_EMPTY), (k - 1) & 1, abort, s.wait_limit_ns)))
                             break;
+                        if (!(ok = mbar_wait(bar(P_FULL + pb), (g >> 1) & 1, abort, s.wait_limit_ns))) break;
                         fence_after_sync();
                         // K step kk (16 keys): 8 TMEM columns of P, 2 KB of the V block
                         const uint32_t a = tmem + kTmemP + pb * 64;
@@ -396,12 +431,12 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
                             for (int kk = 0; kk < 4; ++kk)
                                 mma_ts_split(tmem + kTmemO, a + 32 + kk * 8, b1 + kk * 128, v_hi, id_pv, 1u);
                         }
-                        mma_commit(bar(PV_DONE + pb));
+                        mma_commit(bar(PV_DONE + (g & 3)));
                         mma_commit(bar(V_EMPTY + va));
                         if (!half) mma_commit(bar(V_EMPTY + vb));
                     }
                     if (!ok) break;
-                    mma_commit(bar(O_FULL));
+                    mma_commit(bar(O_FULL + (k & 1)));
                 }
             }
             if (!ok) record_timeout(p, pv ? 5 : 2);
@@ -413,39 +448,45 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
         }
     } else {
         // ------------------------------------------------------------ softmax + epilogue
-        // QN = 128: thread tid owns row tid, keys 0-127 of a tile, d 0-127 of O.
+        // QN = 128: thread wtid owns row wtid, keys 0-127 of a tile, d 0-127 of O.
         // QN = 64: thread (w, lane) owns row 16 w + lane mod 16, keys and d
         // [64 hf, 64 hf + 64) with hf = lane / 16 (its partner is lane ^ 16).
+        if constexpr (QN == 128) regs_inc<208>();
+        const int wg = warp >> 2, quarter = warp & 3, wtid = tid & 127;
         const int hf = QN == 64 ? lane >> 4 : 0;
-        const int row = QN == 64 ? 16 * warp + (lane & 15) : tid;
+        const int row = QN == 64 ? 16 * quarter + (lane & 15) : wtid;
         const float c_log2 = s.sm_scale_log2;
-        const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
+        const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
+        const uint32_t s_addr = tmem + lane_off + kTmemS + wg * 128, p_addr = tmem + lane_off + kTmemP + wg * 64,
+                       o_addr = tmem + lane_off + kTmemO;
         bool ok = true;
         int k = 0;
         for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x, ++k) {
             const int bh = item / nI, qb = item - bh * nI;
             const int32_t* kept = p.kv_idx + (size_t)item * s.n_keep;
-            float neg_m = 0.0f;                      // -m (log2 units)
+            const int g0 = k * T;
+            const int t0 = (g0 & 1) ^ wg;            // this group's first tile of the item (tiles t0, t0 + 2, ...)
+            float neg_m = 0.0f;                      // -m (log2 units) of this row, as this group last used it
             float l0 = 0.0f, l1 = 0.0f, l2 = 0.0f, l3 = 0.0f;
-            int ja_n = __ldg(kept);
-            int jb_n = s.n_keep > 1 ? __ldg(kept + 1) : -1;
-            for (int t = 0; t < T; ++t) {
-                const int g = k * T + t, sb = g & 1;
+            int ja_n = t0 < T ? __ldg(kept + 2 * t0) : 0;
+            int jb_n = 2 * t0 + 1 < s.n_keep ? __ldg(kept + 2 * t0 + 1) : -1;
+            for (int t = t0; t < T; t += 2) {
+                const int g = g0 + t;
                 const int ja = ja_n, jb = jb_n;
-                if (t + 1 < T) {                     // kept ids of the next tile, one tile ahead
-                    ja_n = __ldg(kept + 2 * t + 2);
-                    jb_n = 2 * t + 3 < s.n_keep ? __ldg(kept + 2 * t + 3) : -1;
+                if (t + 2 < T) {                     // kept ids of this group's next tile, one ahead
+                    ja_n = __ldg(kept + 2 * t + 4);
+                    jb_n = 2 * t + 5 < s.n_keep ? __ldg(kept + 2 * t + 5) : -1;
                 }
                 // keys of the pair inside the sequence: block a's first na, block b's first nb
                 const int na = min(64, s.N - ja * 64);
                 const int nb = jb >= 0 ? min(64, s.N - jb * 64) : 0;
-                if (!(ok = mbar_wait(bar(S_FULL + sb), (g >> 1) & 1, abort, s.wait_limit_ns))) break;
+                if (!(ok = mbar_wait(bar(S_FULL + wg), (g >> 1) & 1, abort, s.wait_limit_ns))) break;
                 fence_after_sync();
                 float x[NC];
-                row_load<QN, NC>(tmem + lane_off + kTmemS + sb * 128, x);
+                row_load<QN, NC>(s_addr, x);
                 fence_before_sync();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(S_EMPTY + sb));    // S buffer free for Q K^T(g + 2)
+                if (lane == 0) mbar_arrive(bar(S_EMPTY + wg));    // S buffer free for Q K^T(g + 2)
                 if constexpr (QN == 128) {
                     if (na < 64 || nb < 64) {
 #pragma unroll
@@ -471,36 +512,46 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
                 float tile_max = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
                                        fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
                 if constexpr (QN == 64) tile_max = fmaxf(tile_max, __shfl_xor_sync(0xffffffffu, tile_max, 16));
-                const bool need = t == 0 || fmaf(tile_max, c_log2, neg_m) > kRescaleThreshold;
-                if (__any_sync(0xffffffffu, need)) {
-                    const float neg_m_new = need ? -tile_max * c_log2 : neg_m;
-                    if (t > 0) {
-                        // the O row must hold P V(g - 1) before it is scaled by 2^(m_old - m_new)
-                        const float alpha = fast_exp2(neg_m_new - neg_m);
-                        if (!(ok = mbar_wait(bar(PV_DONE + ((g - 1) & 1)), ((g - 1) >> 1) & 1, abort,
-                                             s.wait_limit_ns)))
-                            break;
-                        fence_after_sync();
-                        const uint32_t oaddr = tmem + lane_off + kTmemO;
-                        // a thread holds as many d columns of its O row as it has keys of a tile
+                // the row's -m after tile g - 1, from the other group's warp of the same rows.  (The
+                // wait is taken at an item's first tile too, where the value has no use: a group
+                // publishes tile g + 1 only after the other has read tile g - 1.)
+                if (g > 0 && !(ok = mbar_wait(bar(M_READY + 4 * (wg ^ 1) + quarter), ((g - 1) >> 1) & 1, abort,
+                                              s.wait_limit_ns)))
+                    break;
+                const float neg_m_prev = t > 0 ? sm.m[wg ^ 1][row] : 0.0f;
+                const bool need = t == 0 || fmaf(tile_max, c_log2, neg_m_prev) > kRescaleThreshold;
+                const float neg_m_new = need ? -tile_max * c_log2 : neg_m_prev;
+                if (hf == 0) sm.m[wg][row] = neg_m_new;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(M_READY + 4 * wg + quarter));
+                // this group's row sum follows m, whoever raised it
+                if (t > 1 && __any_sync(0xffffffffu, neg_m_new != neg_m)) {
+                    const float a = fast_exp2(neg_m_new - neg_m);
+                    l0 *= a;
+                    l1 *= a;
+                    l2 *= a;
+                    l3 *= a;
+                }
+                neg_m = neg_m_new;
+                if (t > 0 && __any_sync(0xffffffffu, need)) {
+                    // the O row must hold P V(g - 1) before it is scaled by 2^(m_old - m_new)
+                    const float alpha = fast_exp2(neg_m_new - neg_m_prev);
+                    if (!(ok = mbar_wait(bar(PV_DONE + ((g - 1) & 3)), ((g - 1) >> 2) & 1, abort, s.wait_limit_ns)))
+                        break;
+                    fence_after_sync();
+                    // a thread holds as many d columns of its O row as it has keys of a tile
 #pragma unroll
-                        for (int c = 0; c < NC / 16; ++c) {
-                            float ov[16];
-                            if constexpr (QN == 128) tmem_ld16(oaddr + c * 16, ov);
-                            else tmem_ld16_half<64>(oaddr + c * 16, ov);
-                            tmem_ld_wait(ov);
+                    for (int c = 0; c < NC / 16; ++c) {
+                        float ov[16];
+                        if constexpr (QN == 128) tmem_ld16(o_addr + c * 16, ov);
+                        else tmem_ld16_half<64>(o_addr + c * 16, ov);
+                        tmem_ld_wait(ov);
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) ov[e] *= alpha;
-                            if constexpr (QN == 128) tmem_st16(oaddr + c * 16, ov);
-                            else tmem_st16_half<64>(oaddr + c * 16, ov);
-                        }
-                        tmem_st_wait();
-                        l0 *= alpha;
-                        l1 *= alpha;
-                        l2 *= alpha;
-                        l3 *= alpha;
+                        for (int e = 0; e < 16; ++e) ov[e] *= alpha;
+                        if constexpr (QN == 128) tmem_st16(o_addr + c * 16, ov);
+                        else tmem_st16_half<64>(o_addr + c * 16, ov);
                     }
-                    neg_m = neg_m_new;
+                    tmem_st_wait();
                 }
                 // p = 2^t, row sum in fp32, P packed to bf16 pairs (lower key in the low half)
                 uint32_t pk[NC / 2];
@@ -520,26 +571,41 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
                     pk[j >> 1] = pack_bf16(p0, p1);
                     pk[(j >> 1) + 1] = pack_bf16(p2, p3);
                 }
-                // P buffer g & 1 is free once P V(g - 2) is done
-                if (g >= 2 && !(ok = mbar_wait(bar(PV_DONE + sb), ((g >> 1) - 1) & 1, abort, s.wait_limit_ns)))
+                // this group's P buffer is free once P V(g - 2) is done
+                if (g >= 2 && !(ok = mbar_wait(bar(PV_DONE + ((g - 2) & 3)), ((g - 2) >> 2) & 1, abort,
+                                               s.wait_limit_ns)))
                     break;
-                row_store<QN, NC / 2>(tmem + lane_off + kTmemP + sb * 64, *reinterpret_cast<const float(*)[NC / 2]>(pk));
+                row_store<QN, NC / 2>(p_addr, *reinterpret_cast<const float(*)[NC / 2]>(pk));
                 tmem_st_wait();
                 fence_before_sync();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(P_FULL + sb));
+                if (lane == 0) mbar_arrive(bar(P_FULL + wg));
             }
             if (!ok) break;
-            // ---- epilogue: O^s row = O / l
             float lsum = (l0 + l1) + (l2 + l3);
             if constexpr (QN == 64) lsum += __shfl_xor_sync(0xffffffffu, lsum, 16);
+            if (((g0 + T - 1) & 1) != wg) {
+                // the other group ends the item: it gets this group's share of the row sums
+                if (T > 1) {
+                    if (hf == 0) sm.l[k & 1][row] = make_float2(lsum, neg_m);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(L_READY + 4 * (k & 1) + quarter));
+                }
+                continue;
+            }
+            // ---- epilogue: O^s row = O / l
+            if (T > 1) {
+                if (!(ok = mbar_wait(bar(L_READY + 4 * (k & 1) + quarter), (k >> 1) & 1, abort, s.wait_limit_ns))) break;
+                const float2 other = sm.l[k & 1][row];
+                lsum = fmaf(other.x, fast_exp2(neg_m - other.y), lsum);
+            }
             const int n = qb * QN + row;
             if (p.lse && hf == 0 && n < s.N) p.lse[(size_t)bh * s.N + n] = (log2f(lsum) - neg_m) * 0.6931471805599453f;
             const float inv_l = 1.0f / lsum;
-            if (!(ok = mbar_wait(bar(O_FULL), k & 1, abort, s.wait_limit_ns))) break;
+            if (!(ok = mbar_wait(bar(O_FULL + (k & 1)), (k >> 1) & 1, abort, s.wait_limit_ns))) break;
             fence_after_sync();
             float ov[NC];                                     // this thread's d columns of the O row
-            row_load<QN, NC>(tmem + lane_off + kTmemO, ov);
+            row_load<QN, NC>(o_addr, ov);
             fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(O_EMPTY));             // O free for the next item's P V
@@ -569,7 +635,7 @@ cudaError_t launch_rows(const Shape& s, const void* qr, const void* kr, const vo
                         void* o_s, float* lse, DeviceStatus* status, cudaStream_t st)
 {
     CUtensorMap mq, mk, mv;
-    if (!make_block_map(&mq, qr, s, QN) || !make_chunk_map(&mk, kr, s) || !make_chunk_map(&mv, v, s))
+    if (!make_block_map(&mq, qr, s, QN) || !make_chunk_map(&mk, kr, s) || !make_block_map(&mv, v, s))
         return cudaErrorInvalidValue;
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
