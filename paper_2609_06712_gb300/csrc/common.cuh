@@ -121,6 +121,16 @@ __device__ __forceinline__ uint32_t slot_mask32(const Shape& s, int b, int c0)
     return s.cube ? slot_mask32_g<true>(s, b, c0) : slot_mask32_g<false>(s, b, c0);
 }
 
+// Cube geometry: bit i tells whether slot 32 hf + i of block b holds a token.  The
+// tokens of a cube form a box, so the mask is built from the box's extents.
+__device__ __forceinline__ uint32_t cube_mask32(const Shape& s, int b, int hf)
+{
+    const CubeOrigin o = cube_origin_rcp(s, b);
+    const int nt = s.T - o.t - 2 * hf, nx = min(4, s.Hh - o.x), ny = min(4, s.Ww - o.y);
+    const uint32_t plane = (0x1111u * ((1u << ny) - 1u)) & ((1u << (4 * nx)) - 1u);     // 4 rows of 4 slots
+    return (nt > 0 ? plane : 0u) | (nt > 1 ? plane << 16 : 0u);
+}
+
 // Rotation (cos, sin) of pair m for the token at flat index n.
 __device__ __forceinline__ float2 rope_cs(const float2* __restrict__ tab, const Shape& s, int n, int m)
 {

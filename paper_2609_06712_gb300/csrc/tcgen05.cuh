@@ -262,6 +262,65 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16])
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
 
+// D[tmem] (+)= A[tmem] * B[smem]: A is M rows of K 16-bit values in TMEM,
+// two per 32-bit column (the lower K index in the low half).
+__device__ __forceinline__ void mma_ts_split(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi,
+                                             uint32_t idesc, uint32_t accum)
+{
+    asm volatile(
+        "{\n.reg .pred p;\n.reg .b64 db;\n"
+        "setp.ne.b32 p, %5, 0;\n"
+        "mov.b64 db, {%2, %3};\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n}\n" ::"r"(d_tmem),
+        "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accum)
+        : "memory");
+}
+
+// 16x32bx2 accesses: over the 16 lanes from taddr's lane, threads 0-15 take
+// lane `lane` at columns [c, c + 16), threads 16-31 lane `lane - 16` at
+// columns [c + OFF, c + OFF + 16).
+template <int OFF>
+__device__ __forceinline__ void tmem_ld16_half(uint32_t taddr, float (&v)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x32bx2.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16], %17;\n"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
+          "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+        : "r"(taddr), "n"(OFF));
+}
+template <int OFF>
+__device__ __forceinline__ void tmem_st16_half(uint32_t taddr, const float (&v)[16])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.16x32bx2.x16.b32 [%0], %17, {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n" ::"r"(
+            taddr),
+        "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
+        "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]), "n"(OFF)
+        : "memory");
+}
+
+// (a, b) = (a * m + c, b * m + c), one packed f32x2 instruction (each element an IEEE fma)
+__device__ __forceinline__ void ffma2(float& a, float& b, float m, float c)
+{
+    asm("{\n.reg .b64 ra, rm, rc;\nmov.b64 ra, {%0, %1};\nmov.b64 rm, {%2, %2};\nmov.b64 rc, {%3, %3};\n"
+        "fma.rn.f32x2 ra, ra, rm, rc;\nmov.b64 {%0, %1}, ra;\n}\n"
+        : "+f"(a), "+f"(b) : "f"(m), "f"(c));
+}
+__device__ __forceinline__ void fadd2(float& a, float& b, float p, float q)
+{
+    asm("{\n.reg .b64 ra, rp;\nmov.b64 ra, {%0, %1};\nmov.b64 rp, {%2, %3};\n"
+        "add.rn.f32x2 ra, ra, rp;\nmov.b64 {%0, %1}, ra;\n}\n"
+        : "+f"(a), "+f"(b) : "f"(p), "f"(q));
+}
+
+// (a, b) *= (p, q)
+__device__ __forceinline__ void fmul2(float& a, float& b, float p, float q)
+{
+    asm("{\n.reg .b64 ra, rp;\nmov.b64 ra, {%0, %1};\nmov.b64 rp, {%2, %3};\n"
+        "mul.rn.f32x2 ra, ra, rp;\nmov.b64 {%0, %1}, ra;\n}\n"
+        : "+f"(a), "+f"(b) : "f"(p), "f"(q));
+}
+
 // barrier.cta.red.or over `count` threads on named barrier `id`.
 __device__ __forceinline__ bool bar_red_or(int id, int count, bool pred)
 {
