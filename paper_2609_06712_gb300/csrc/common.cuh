@@ -88,9 +88,7 @@ __host__ __device__ __forceinline__ int cube_token(const Shape& s, CubeOrigin o,
 }
 
 // Either geometry: the token of slot i of block b (-1 for a slot past the
-// sequence or outside the grid), and the validity of the 32 slots [c0, c0 + 32)
-// of block b as a bit mask.
-// (The template forms fix the geometry at compile time.)
+// sequence or outside the grid).  (The template form fixes the geometry at compile time.)
 template <bool kCube>
 __device__ __forceinline__ int slot_token_g(const Shape& s, int b, int i)
 {
@@ -101,26 +99,6 @@ __device__ __forceinline__ int slot_token(const Shape& s, int b, int i)
 {
     return s.cube ? slot_token_g<true>(s, b, i) : slot_token_g<false>(s, b, i);
 }
-template <bool kCube>
-__device__ __forceinline__ uint32_t slot_mask32_g(const Shape& s, int b, int c0)
-{
-    if constexpr (!kCube) {
-        const int rem = s.N - b * 64 - c0;
-        return rem >= 32 ? 0xffffffffu : (rem <= 0 ? 0u : (1u << rem) - 1u);
-    }
-    else {
-        const CubeOrigin o = cube_origin_rcp(s, b);
-        uint32_t m = 0;
-        for (int i = 0; i < 32; ++i)
-            if (cube_token(s, o, c0 + i) >= 0) m |= 1u << i;
-        return m;
-    }
-}
-__device__ __forceinline__ uint32_t slot_mask32(const Shape& s, int b, int c0)
-{
-    return s.cube ? slot_mask32_g<true>(s, b, c0) : slot_mask32_g<false>(s, b, c0);
-}
-
 // Cube geometry: bit i tells whether slot 32 hf + i of block b holds a token.  The
 // tokens of a cube form a box, so the mask is built from the box's extents.
 __device__ __forceinline__ uint32_t cube_mask32(const Shape& s, int b, int hf)
@@ -129,6 +107,18 @@ __device__ __forceinline__ uint32_t cube_mask32(const Shape& s, int b, int hf)
     const int nt = s.T - o.t - 2 * hf, nx = min(4, s.Hh - o.x), ny = min(4, s.Ww - o.y);
     const uint32_t plane = (0x1111u * ((1u << ny) - 1u)) & ((1u << (4 * nx)) - 1u);     // 4 rows of 4 slots
     return (nt > 0 ? plane : 0u) | (nt > 1 ? plane << 16 : 0u);
+}
+
+// Either geometry: bit i tells whether slot 32 hf + i of block b holds a token (b < 0: none does).
+template <bool kCube>
+__device__ __forceinline__ uint32_t block_mask32(const Shape& s, int b, int hf)
+{
+    if (b < 0) return 0u;
+    if constexpr (kCube) return cube_mask32(s, b, hf);
+    else {
+        const int rem = s.N - b * 64 - 32 * hf;
+        return rem >= 32 ? 0xffffffffu : (rem <= 0 ? 0u : (1u << rem) - 1u);
+    }
 }
 
 // Rotation (cos, sin) of pair m for the token at flat index n.
@@ -176,8 +166,8 @@ struct Workspace {
 
 // Host launchers, one per kernel family.  All return cudaGetLastError().
 cudaError_t launch_rope_table(const rola_config_t& cfg, float2* tab, cudaStream_t st);
-// q^r, k^r (rows in block order, Np per head) and the block means; in cube
-// geometry also v copied into block order (vp) when v is given.  With
+// q^r, k^r (rows in block order, Np per head) and the block means, each only
+// where its pointer is given; in cube geometry also v copied into block order (vp) when v is given.  With
 // 128-token query blocks (s.qb2) qbar receives the 64-token blocks' q SUMS,
 // which launch_qpool128 turns into the 128-token means.
 cudaError_t launch_rope_pool(const rola_config_t& cfg, const Shape& s, const void* q, const void* k,
@@ -192,9 +182,6 @@ cudaError_t launch_qpool128(const Shape& s, const float* qsum64, float* qbar128,
 cudaError_t launch_sparse_attn(rola_dtype_t dt, const Shape& s, const void* qr, const void* kr,
                                const void* v, const int32_t* kv_idx, void* o_s, float* lse, DeviceStatus* status,
                                cudaStream_t st);
-cudaError_t launch_sparse_attn_tc(const Shape& s, const void* qr, const void* kr, const void* v,
-                                  const int32_t* kv_idx, void* o_s, float* lse, DeviceStatus* status,
-                                  cudaStream_t st);
 cudaError_t launch_lowrank_summary(rola_dtype_t dt, const Shape& s, int nsplit, const void* k,
                                    const void* v, const void* P_k, const float2* tab, float* partials,
                                    float* C, float* z, __nv_bfloat16* Cbf, cudaStream_t st);

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kF32Threads) sparse_attn_f32_kernel(Shape s, c
     }
 }
 
-// bf16 with contiguous key blocks (sparse_attn_rows.cu)
+// bf16 (sparse_attn_rows.cu)
 cudaError_t launch_sparse_attn_rows(const Shape& s, const void* qr, const void* kr, const void* v,
                                     const int32_t* kv_idx, void* o_s, float* lse, DeviceStatus* status,
                                     cudaStream_t st);
@@ -110,8 +110,7 @@ cudaError_t launch_sparse_attn_rows(const Shape& s, const void* qr, const void* 
 cudaError_t launch_sparse_attn(rola_dtype_t dt, const Shape& s, const void* qr, const void* kr, const void* v,
                                const int32_t* kv_idx, void* o_s, float* lse, DeviceStatus* status, cudaStream_t st)
 {
-    if (dt == ROLA_BF16 && !s.cube) return launch_sparse_attn_rows(s, qr, kr, v, kv_idx, o_s, lse, status, st);
-    if (dt == ROLA_BF16) return launch_sparse_attn_tc(s, qr, kr, v, kv_idx, o_s, lse, status, st);
+    if (dt == ROLA_BF16) return launch_sparse_attn_rows(s, qr, kr, v, kv_idx, o_s, lse, status, st);
     dim3 grid(s.nB, s.B * s.H);
     size_t smem = sizeof(float) * (2 * kBlock * kPad + kBlock * kDh + kBlock * 65);
     cudaError_t e = cudaFuncSetAttribute(sparse_attn_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -5,7 +5,10 @@
 //
 // (Sec. 3 softmax form restricted to the kept key blocks, Alg. 1 sparse
 // branch.)  Query blocks of QN = 64 tokens (the mask of Alg. 1) or QN = 128
-// tokens (a mask chosen per 128-token chunk); key blocks are 64 tokens.
+// tokens (a mask chosen per 128-token chunk); key blocks are 64 tokens.  With
+// cube blocks (kCube) q^r, k^r and v come in block order, 64 slots a cube, so a
+// cube is one box like a chunk; empty slots are masked out of the softmax and
+// each O^s row goes to its slot's token.
 //
 // An item (one query block of one head) is the M = QN rows of tcgen05 MMAs:
 //   S    = Q (QN q x 128 d, smem, K-major)  x  K_pair^T (N = 128 keys, smem, K-major)
@@ -58,6 +61,8 @@
 //     the next block ids in registers needs ~350 for two boxes.  14.76 -> 11.85
 //     ms (QN = 64); the L2 itself delivers a 16 KB block per 248 cycles and SM.
 //   - two softmax groups in turn: 11.85 -> 11.5 ms (QN = 64), 8.2 -> 7.3 ms (QN = 128).
+//   - cube blocks on this kernel instead of a transposed form of their own: 4.88 ->
+//     3.43 ms (40 heads, 21 x 30 x 52 grid, 62 of 624 cubes kept).
 //   - QN = 64 now takes 1137 cycles a tile: 1024 of tensor work (an M = 64
 //     product runs at half the M = 128 rate) and 144 KB through the shared
 //     memory (1125 at 128 B/cycle).  QN = 128 takes ~1400 cycles against the
@@ -171,7 +176,7 @@ __device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.a
 template <int R>
 __device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(R)); }
 
-template <int QN>
+template <int QN, bool kCube>
 __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __grid_constant__ CUtensorMap map_q,
                                                                        const __grid_constant__ CUtensorMap map_k,
                                                                        const __grid_constant__ CUtensorMap map_v,
@@ -426,9 +431,6 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
                     ja_n = __ldg(kept + 2 * t + 4);
                     jb_n = 2 * t + 5 < s.n_keep ? __ldg(kept + 2 * t + 5) : -1;
                 }
-                // keys of the pair inside the sequence: block a's first na, block b's first nb
-                const int na = min(64, s.N - ja * 64);
-                const int nb = jb >= 0 ? min(64, s.N - jb * 64) : 0;
                 if (!(ok = mbar_wait(bar(S_FULL + wg), (g >> 1) & 1, abort, s.wait_limit_ns))) break;
                 fence_after_sync();
                 float x[NC];
@@ -436,7 +438,10 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
                 fence_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(S_EMPTY + wg));    // S buffer free for Q K^T(g + 2)
+                // keys of the tile that are tokens; the others (a ragged block's end, an edge cube's empty
+                // slots, the absent second block of a half tile) drop out of the maximum and the sum
                 if constexpr (QN == 128) {
+                    const int na = min(64, s.N - ja * 64), nb = jb >= 0 ? min(64, s.N - jb * 64) : 0;
                     if (na < 64 || nb < 64) {
 #pragma unroll
                         for (int j = 0; j < 64; ++j) {
@@ -445,11 +450,17 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
                         }
                     }
                 } else {
-                    const int nv = hf ? nb : na;
-                    if (nv < 64) {
+                    const int blk = hf ? jb : ja;
+                    const int left = blk >= 0 ? s.N - blk * 64 : 0;           // chunks: tokens from the block on
+                    if (kCube || left < 64) {
+                        const uint32_t m0 = block_mask32<kCube>(s, blk, 0), m1 = block_mask32<kCube>(s, blk, 1);
+                        if (!kCube || (m0 & m1) != 0xffffffffu) {
 #pragma unroll
-                        for (int j = 0; j < 64; ++j)
-                            if (j >= nv) x[j] = -INFINITY;
+                            for (int j = 0; j < 32; ++j) {
+                                if (!((m0 >> j) & 1u)) x[j] = -INFINITY;
+                                if (!((m1 >> j) & 1u)) x[32 + j] = -INFINITY;
+                            }
+                        }
                     }
                 }
                 // the tile's row maximum (eight independent chains; the two halves of a row meet by shuffle)
@@ -548,8 +559,8 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
                 const float2 other = sm.l[k & 1][row];
                 lsum = fmaf(other.x, fast_exp2(neg_m - other.y), lsum);
             }
-            const int n = qb * QN + row;
-            if (p.lse && hf == 0 && n < s.N) p.lse[(size_t)bh * s.N + n] = (log2f(lsum) - neg_m) * 0.6931471805599453f;
+            const int n = kCube ? slot_token_g<kCube>(s, qb, row) : (qb * QN + row < s.N ? qb * QN + row : -1);
+            if (p.lse && hf == 0 && n >= 0) p.lse[(size_t)bh * s.N + n] = (log2f(lsum) - neg_m) * 0.6931471805599453f;
             const float inv_l = 1.0f / lsum;
             if (!(ok = mbar_wait(bar(O_FULL + (k & 1)), (k >> 1) & 1, abort, s.wait_limit_ns))) break;
             fence_after_sync();
@@ -558,7 +569,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
             fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(O_EMPTY));             // O free for the next item's P V
-            if (n < s.N) {
+            if (n >= 0) {
                 uint4* dst = reinterpret_cast<uint4*>(p.o + ((size_t)bh * s.N + n) * kDh + hf * 64);
 #pragma unroll
                 for (int c = 0; c < NC / 8; ++c) {
@@ -579,12 +590,15 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
     if (warp == kMmaWarp) tmem_dealloc(tmem, kTmemCols);
 }
 
-template <int QN>
+template <int QN, bool kCube>
 cudaError_t launch_rows(const Shape& s, const void* qr, const void* kr, const void* v, const int32_t* kv_idx,
                         void* o_s, float* lse, DeviceStatus* status, cudaStream_t st)
 {
+    // the maps span the block-ordered rows (the token order itself for contiguous chunks)
+    Shape rows = s;
+    rows.N = s.Np;
     CUtensorMap mq, mk, mv;
-    if (!make_block_map(&mq, qr, s, QN) || !make_chunk_map(&mk, kr, s) || !make_block_map(&mv, v, s))
+    if (!make_block_map(&mq, qr, rows, QN) || !make_chunk_map(&mk, kr, rows) || !make_block_map(&mv, v, rows))
         return cudaErrorInvalidValue;
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -602,23 +616,23 @@ cudaError_t launch_rows(const Shape& s, const void* qr, const void* kr, const vo
     p.tiles = (s.n_keep + 1) / 2;
     const size_t smem = Cfg<QN>::kSmemTiles + sizeof(Ctrl<QN>);
     const int grid = p.total_items < nsm ? p.total_items : nsm;
-    e = cudaFuncSetAttribute(sparse_attn_rows_kernel<QN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kernel = sparse_attn_rows_kernel<QN, kCube>;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    sparse_attn_rows_kernel<QN><<<grid, kThreads, smem, st>>>(mq, mk, mv, p);
+    kernel<<<grid, kThreads, smem, st>>>(mq, mk, mv, p);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-// Contiguous 64-token key blocks; 64-token query blocks (s.qb2 == 0, the mask
-// has nQ = nB rows) or 128-token query chunks (s.qb2 == 1).
+// 64-token key blocks; query blocks of 64 slots (chunks or cubes; the mask has
+// nQ = nB rows) or, with chunks, of 128 tokens (s.qb2 == 1).
 cudaError_t launch_sparse_attn_rows(const Shape& s, const void* qr, const void* kr, const void* v,
                                     const int32_t* kv_idx, void* o_s, float* lse, DeviceStatus* status,
                                     cudaStream_t st)
 {
-    if (s.cube) return cudaErrorInvalidValue;
-    return s.qb2 ? launch_rows<128>(s, qr, kr, v, kv_idx, o_s, lse, status, st)
-                 : launch_rows<64>(s, qr, kr, v, kv_idx, o_s, lse, status, st);
+    auto launch = s.cube ? launch_rows<64, true> : (s.qb2 ? launch_rows<128, false> : launch_rows<64, false>);
+    return launch(s, qr, kr, v, kv_idx, o_s, lse, status, st);
 }
 
 }  // namespace rola

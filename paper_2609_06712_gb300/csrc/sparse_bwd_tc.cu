@@ -141,15 +141,6 @@ __device__ __forceinline__ void mma_grad(uint32_t d, uint32_t a, uint32_t gap, u
     for (int kk = 0; kk < 4; ++kk) mma_ts_split(d, a + gap + kk * 8, b + (kk + 4) * 128, b_hi, id, 1u);
 }
 
-// Bit i: slot 32 hf + i of block b holds a token (b < 0: none does).
-template <bool kCube>
-__device__ __forceinline__ uint32_t half_mask(const Shape& s, int b, int hf)
-{
-    if (b < 0) return 0u;
-    if constexpr (kCube) return cube_mask32(s, b, hf);
-    else return slot_mask32_g<false>(s, b, 32 * hf);
-}
-
 // The 32 outputs of a thread (columns d0 .. d0 + 31 of one row) at dst, as bf16.
 __device__ __forceinline__ void store_row32(__nv_bfloat16* dst, const float (&v)[kCols])
 {
@@ -372,7 +363,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
             for (int t = 0; t < T; ++t, ++g) {
                 const int j = j_n;
                 if (t + 1 < T) j_n = 2 * t + 2 + wg < s.n_keep ? __ldg(kept + 2 * t + 2 + wg) : -1;
-                const uint32_t keys = half_mask<kCube>(s, j, hf);       // columns that are tokens
+                const uint32_t keys = block_mask32<kCube>(s, j, hf);       // columns that are tokens
                 if (!(ok = mbar_wait(bar(S_FULL), g & 1, abort, s.wait_limit_ns))) break;
                 fence_after_sync();
                 float x[kCols], y[kCols];
