@@ -4,20 +4,21 @@
 //   r_p    = sqrt(mean_i (O^s_{p,i})^2 + eps_fuse)
 //   O_p    = O^s_p + g_p r_p O^lr_p                     Eq. (gate), (O^s/r_p + g O^lr) r_p
 //
-// Work unit = (head, 64-token block); G persistent CTAs (two per SM for
-// r <= 48, else one) take
-// contiguous unit ranges, so P_q and C (bf16) are loaded once per head a CTA
-// meets instead of once per block.  Each unit's q and O^s blocks arrive by TMA
-// (one 16 KB [chunk][row][64] box each) in a ring of stages; the fused O is
-// written over O^s in the stage and leaves by a TMA store, which also clips
-// the rows past N of the last block.  The loads of unit i + S - 1 go out after
-// unit i's first barrier, once the store that last read that stage is done
-// reading it.
-//
-// Eight warps per unit: warp w takes tokens 16 (w & 3) .. +15 and half h = w >> 2
-// of the work: U = Q P_q^T for half of the r columns (then q~ to shared
-// memory), y = q~ C for d in [64 h, 64 h + 64); the row sums of y^2 and of
-// (O^s)^2 are combined over the two halves through shared memory.
+// Work unit = (head, 16-token tile).  One persistent CTA per SM takes a contiguous
+// range of tiles; P_q and C (bf16) are loaded once per head it meets, and within a
+// head every warp works on tiles of its own with no barrier between warps:
+//   U = Q P_q^T (mma.sync), q~ = R_r SiLU(U) in registers
+//   (an accumulator pair is the A fragment of the next product), y += q~ C for all
+//   128 d, the row sums of y^2 and (O^s)^2 over the four lanes of a row, and O
+//   written over O^s in shared memory, from where a TMA store takes it (which also
+//   clips the rows past N).
+// A warp owns a q buffer (refilled as soon as its fragments are in registers) and
+// two O^s buffers (one for r > 64), filled by its own TMA loads, so the warps of an
+// SM are at different points of the chain and their loads, products and stores
+// overlap.  Bound by HBM: 768 B per (head, token).  720p layer (40 heads, 75600
+// tokens): r = 32 496 -> 440 us (5.3 TB/s), r = 64 1048 -> 624 us; the form before
+// (64-token units over 8 warps with three CTA barriers each, one or two CTAs an SM)
+// waited on its own chain most of the time.
 #include <cudaTypedefs.h>
 
 #include "common.cuh"
@@ -29,32 +30,26 @@ namespace {
 
 using namespace tc;
 
-constexpr int kWarps = 8;
-constexpr int kThreads = 32 * kWarps;
-constexpr uint32_t kBox = 64 * 128 * 2;
-constexpr int kMaxStages = 4;
-
-// r <= 48: two CTAs per SM (16 warps) with a 2-deep ring; wider r: one CTA
-// with a 4-deep ring (P_q and C take more shared memory and registers)
-template <int R>
-struct Occupancy {
-    static constexpr int ctas = R <= 48 ? 2 : 1;
-    static constexpr int stages = R <= 48 ? 2 : 4;
-};
+constexpr int kTile = 16;                            // tokens of a tile
+constexpr uint32_t kBox = kTile * 128 * 2;           // [chunk][16 rows][64]
 
 template <int R>
 struct Layout {
-    static constexpr int NT = R / 8;
-    static constexpr int NTW = NT / 2;               // n-tiles of U per warp
-    static constexpr int QT = 2 * R + 16;            // bytes per q~ row (padded against bank conflicts)
-    static constexpr uint32_t stage_bytes = 2 * kBox;   // q | O^s
-    static constexpr uint32_t P = Occupancy<R>::stages * stage_bytes;
+    static constexpr int warps = R <= 64 ? 16 : 12;  // (registers: 128 or 168 a thread)
+    static constexpr int OB = R <= 64 ? 2 : 1;       // O^s buffers of a warp
+    static constexpr uint32_t warp_bytes = (1 + OB) * kBox;     // q | O^s ...
+    static constexpr uint32_t P = warps * warp_bytes;
     static constexpr uint32_t C = P + R * 256;
-    static constexpr uint32_t qt = C + R * 256;
-    static constexpr uint32_t red = qt + 64 * QT;    // [y^2 | O^s^2][half][64 rows] fp32
-    static constexpr uint32_t bars = red + 2 * 2 * 64 * 4;
-    static constexpr uint32_t total = bars + kMaxStages * 8 + 16;
+    static constexpr uint32_t bars = C + R * 256;    // full barriers of every warp: q, O^s ...
+    static constexpr uint32_t abort = bars + warps * (1 + OB) * 8;
+    static constexpr uint32_t total = abort + 16;
 };
+
+// Byte offset of 16-byte chunk c (0..15) of row r in a 16-row box (128-byte swizzle).
+__device__ __forceinline__ uint32_t wsw(int r, int c)
+{
+    return (c >> 3) * (kTile * 128) + r * 128 + (((c & 7) ^ (r & 7)) << 4);
+}
 
 struct Params {
     Shape s;
@@ -63,7 +58,7 @@ struct Params {
     const float* gate;
     const float2* tab;
     DeviceStatus* status;
-    int units;
+    int tiles;                // 16-token tiles of a head
 };
 
 // SiLU with the MUFU exponential; the kernel is instantiated for it and for
@@ -74,71 +69,66 @@ struct SiluMufu {
 };
 
 template <int R, typename Act>
-__global__ void __launch_bounds__(kThreads, Occupancy<R>::ctas) readout_kernel(const __grid_constant__ CUtensorMap map_q,
-                                                              const __grid_constant__ CUtensorMap map_os,
-                                                              const __grid_constant__ CUtensorMap map_o,
-                                                              const Params p)
+__global__ void __launch_bounds__(32 * Layout<R>::warps, 1) readout_kernel(const __grid_constant__ CUtensorMap map_q,
+                                                                          const __grid_constant__ CUtensorMap map_os,
+                                                                          const __grid_constant__ CUtensorMap map_o,
+                                                                          const Params p)
 {
     using L = Layout<R>;
-    constexpr int NTW = L::NTW;
-    constexpr int kStages = Occupancy<R>::stages;
+    constexpr int kWarps = L::warps, kThreads = 32 * kWarps, OB = L::OB;
     extern __shared__ __align__(1024) uint8_t smem[];
     if (smem_u32(smem) & 1023u) {
         if (threadIdx.x == 0) atomicCAS(&p.status->code, 0, (int)ROLA_ERR_UNSUPPORTED);
         return;
     }
     const Shape& s = p.s;
-    const uint32_t sbase = smem_u32(smem), sP = sbase + L::P, sC = sbase + L::C, sQt = sbase + L::qt;
-    float* red = reinterpret_cast<float*>(smem + L::red);
-    const uint32_t full0 = sbase + L::bars;
-    volatile int* abort = reinterpret_cast<volatile int*>(smem + L::bars + kMaxStages * 8);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t4 = lane & 3, mi = lane >> 3;
-    const int mt = warp & 3, half = warp >> 2;
-    const int u0 = (int)((long long)blockIdx.x * p.units / gridDim.x);
-    const int u1 = (int)((long long)(blockIdx.x + 1) * p.units / gridDim.x);
-    const int count = u1 - u0;
+    const uint32_t sbase = smem_u32(smem), sP = sbase + L::P, sC = sbase + L::C;
+    const uint32_t qb = sbase + warp * L::warp_bytes;
+    const uint32_t q_full = sbase + L::bars + warp * (1 + OB) * 8, o_full = q_full + 8;
+    volatile int* abort = reinterpret_cast<volatile int*>(smem + L::abort);
+    const long long total = (long long)s.B * s.H * p.tiles;
+    const long long u0 = (long long)blockIdx.x * total / gridDim.x, u1 = (long long)(blockIdx.x + 1) * total / gridDim.x;
+    const int hw = s.Hh * s.Ww;
 
     if (tid == 0) {
         *abort = 0;
-        for (int i = 0; i < kStages; ++i) mbar_init(full0 + 8 * i, 1);
+        for (int i = 0; i < kWarps * (1 + OB); ++i) mbar_init(sbase + L::bars + 8 * i, 1);
         fence_mbar_init();
         tma_prefetch_desc(&map_q);
         tma_prefetch_desc(&map_os);
         tma_prefetch_desc(&map_o);
     }
-    __syncthreads();
-
-    // loads of the j-th unit into stage j % S, by thread 0 (the thread that
-    // stores, so that its bulk-group waits order a refill after the store)
-    auto issue = [&](int j) {
-        const int u = u0 + j, bh = u / s.nC, blk = u - bh * s.nC, st = j % kStages;
-        const uint32_t dst = sbase + st * L::stage_bytes, bar = full0 + 8 * st;
-        if (tid == 0) {
-            mbar_expect_tx(bar, 2 * kBox);
-            tma_load_4d(dst, &map_q, bar, 0, blk * 64, 0, bh);
-            tma_load_4d(dst + kBox, &map_os, bar, 0, blk * 64, 0, bh);
+    bool ok = true;
+    int i = 0;                                       // tiles of this warp so far (buffer and phase)
+    int q_issued = 0, o_issued = 0;                  // loads of this warp so far
+    for (long long u = u0; u < u1;) {
+        const int bh = (int)(u / p.tiles), first = (int)(u - (long long)bh * p.tiles);
+        const int end = (int)min((long long)p.tiles, first + (u1 - u));
+        u += end - first;
+        // (lane 0 issues all of a warp's copies, so that its bulk-group waits order a refill after the store)
+        auto load_q = [&](int x) {
+            if (lane == 0) {
+                mbar_expect_tx(q_full, kBox);
+                tma_load_4d(qb, &map_q, q_full, 0, x * kTile, 0, bh);
+            }
+            ++q_issued;
+        };
+        auto load_o = [&](int x, int buf) {
+            if (lane == 0) {
+                bulk_wait_read_all();                // the store that last read the buffer
+                mbar_expect_tx(o_full + 8 * buf, kBox);
+                tma_load_4d(qb + kBox + buf * kBox, &map_os, o_full + 8 * buf, 0, x * kTile, 0, bh);
+            }
+            ++o_issued;
+        };
+        __syncthreads();                             // the barriers are initialised; every reader of the last head is done
+        if (ok && first + warp < end) {
+            load_q(first + warp);
+            load_o(first + warp, i % OB);
         }
-    };
-    int issued = count < kStages ? count : kStages;
-    for (int j = 0; j < issued; ++j) issue(j);
-
-    int kaxis[NTW];
-#pragma unroll
-    for (int j = 0; j < NTW; ++j) {
-        const int m = (half * NTW + j) * 4 + t4;
-        kaxis[j] = m < s.pt ? 0 : (m < s.pt + s.px ? 1 : 2);
-    }
-    const int hw = s.Hh * s.Ww;
-
-    int hb = -1;
-    bool failed = false;
-    int i = 0;
-    for (int u = u0; u < u1; ++u, ++i) {
-        const int bh = u / s.nC, blk = u - bh * s.nC, b = bh / s.H;
-        const int st = i % kStages;
-        if (bh != hb) {
-            // P_q of the head and C of (batch, head); every reader of the old ones has passed the last barrier
+        {
             const uint4* srcP = reinterpret_cast<const uint4*>(p.Pq + (size_t)(bh % s.H) * s.r * kDh);
             const uint4* srcC = reinterpret_cast<const uint4*>(p.Cbf + (size_t)bh * R * kDh);   // rp rows
             for (int e = tid; e < R * 16; e += kThreads) {
@@ -151,175 +141,124 @@ __global__ void __launch_bounds__(kThreads, Occupancy<R>::ctas) readout_kernel(c
                              "r"(c.w)
                              : "memory");
             }
-            bar_sync(1, kThreads);
-            hb = bh;
         }
-        const uint32_t qb = sbase + st * L::stage_bytes, ob = qb + kBox;
-        const int n_base = blk * kBlock;
-        // (cos, sin) of this thread's q~ pairs for its two tokens
-        float2 kcs[2][NTW];
-        {
-            const int n = n_base + mt * 16 + g;
-            int t = n / hw;
-            const int rem = n - t * hw;
-            int x = rem / s.Ww, y = rem - x * s.Ww;
+        __syncthreads();
+        // a warp whose wait gave up stays for the barriers of the heads to come and works no further tile
+        for (int x = first + warp; ok && x < end; x += kWarps, ++i) {
+            const int buf = i % OB;
+            const bool more = x + kWarps < end;
+            if (OB == 2 && more) load_o(x + kWarps, buf ^ 1);
+            // grid positions and gates of this thread's two tokens
+            const int n_lo = x * kTile + g;
+            int tt[2], xx[2], yy[2];
+            float gp[2];
 #pragma unroll
             for (int hr = 0; hr < 2; ++hr) {
-#pragma unroll
-                for (int j = 0; j < NTW; ++j) {
-                    const int row = kaxis[j] == 0 ? min(t, s.T - 1) : (kaxis[j] == 1 ? s.T + x : s.T + s.Hh + y);
-                    kcs[hr][j] = __ldg(p.tab + row * kPairs + (half * NTW + j) * 4 + t4);
-                }
-                y += 8;
-                while (y >= s.Ww) {
-                    y -= s.Ww;
-                    if (++x == s.Hh) {
-                        x = 0;
-                        ++t;
-                    }
-                }
+                const int n = min(n_lo + 8 * hr, s.N - 1);
+                tt[hr] = n / hw;
+                const int rem = n - tt[hr] * hw;
+                xx[hr] = rem / s.Ww;
+                yy[hr] = rem - xx[hr] * s.Ww;
+                gp[hr] = p.gate ? __ldg(p.gate + (size_t)(bh / s.H) * s.N + n) : s.default_gate;
             }
-        }
-        // the gate of this thread's two rows, loaded ahead of use
-        const int r_lo = mt * 16 + g, r_hi = r_lo + 8;
-        float gp[2];
+            ok = __all_sync(0xffffffffu, mbar_wait(q_full, i & 1, abort, s.wait_limit_ns));
+            if (!ok) break;
+            // ---- U = Q P_q^T, all r columns
+            float u[R / 8][4];
 #pragma unroll
-        for (int hr = 0; hr < 2; ++hr) {
-            const int n = min(n_base + (hr ? r_hi : r_lo), s.N - 1);
-            gp[hr] = p.gate ? __ldg(p.gate + (size_t)b * s.N + n) : s.default_gate;
-        }
-        const bool ok = mbar_wait(full0 + 8 * st, (i / kStages) & 1, abort, s.wait_limit_ns);
-        if (ok) {
-            // ---- U = Q P_q^T: tokens 16 mt .. +15, this warp's half of the r columns
-            float uacc[NTW][4];
-#pragma unroll
-            for (int j = 0; j < NTW; ++j) uacc[j][0] = uacc[j][1] = uacc[j][2] = uacc[j][3] = 0.0f;
+            for (int j = 0; j < R / 8; ++j) u[j][0] = u[j][1] = u[j][2] = u[j][3] = 0.0f;
 #pragma unroll
             for (int kc = 0; kc < 8; ++kc) {
                 uint32_t a0, a1, a2, a3;
-                ldsm_x4(qb + tsw(mt * 16 + (lane & 7) + (mi & 1) * 8, kc * 2 + (mi >> 1)), a0, a1, a2, a3);
+                ldsm_x4(qb + wsw((lane & 7) + (mi & 1) * 8, kc * 2 + (mi >> 1)), a0, a1, a2, a3);
 #pragma unroll
-                for (int np = 0; np < NTW / 2; ++np) {
-                    const int nt = half * NTW + 2 * np;
+                for (int j = 0; j < R / 16; ++j) {
                     uint32_t b0, b1, b2, b3;
-                    ldsm_x4(sP + sw128(nt * 8 + (mi >> 1) * 8 + (lane & 7), kc * 2 + (mi & 1)), b0, b1, b2, b3);
-                    mma_bf16(uacc[2 * np], a0, a1, a2, a3, b0, b1);
-                    mma_bf16(uacc[2 * np + 1], a0, a1, a2, a3, b2, b3);
-                }
-                if (NTW & 1) {
-                    const int nt = half * NTW + NTW - 1;
-                    uint32_t b0, b1;
-                    ldsm_x2(sP + sw128(nt * 8 + (lane & 7), kc * 2 + (mi & 1)), b0, b1);
-                    mma_bf16(uacc[NTW - 1], a0, a1, a2, a3, b0, b1);
+                    ldsm_x4(sP + sw128(j * 16 + (mi >> 1) * 8 + (lane & 7), kc * 2 + (mi & 1)), b0, b1, b2, b3);
+                    mma_bf16(u[2 * j], a0, a1, a2, a3, b0, b1);
+                    mma_bf16(u[2 * j + 1], a0, a1, a2, a3, b2, b3);
                 }
             }
-            // ---- q~ (bf16) into shared memory; tokens past N give zero features
+            __syncwarp();
+            if (more) load_q(x + kWarps);
+            // ---- q~: an accumulator's two rows and column pair are the A fragment of the next product
+            // (rows of tokens past N are never stored)
+            uint32_t af[R / 8][2];
+#pragma unroll
+            for (int j = 0; j < R / 8; ++j)
+#pragma unroll
+                for (int hr = 0; hr < 2; ++hr) {
+                    const int m = j * 4 + t4;
+                    const int row = m < s.pt ? tt[hr] : (m < s.pt + s.px ? s.T + xx[hr] : s.T + s.Hh + yy[hr]);
+                    const float2 f = lowrank_pair(u[j][2 * hr], u[j][2 * hr + 1], __ldg(p.tab + row * kPairs + m),
+                                                  s.lr_rope, Act{s.lr_act});
+                    af[j][hr] = pack_bf16(f.x, f.y);
+                }
+            // ---- y = q~ C
+            float y[16][4];
+#pragma unroll
+            for (int d = 0; d < 16; ++d) y[d][0] = y[d][1] = y[d][2] = y[d][3] = 0.0f;
+#pragma unroll
+            for (int j = 0; j < R / 16; ++j)
+#pragma unroll
+                for (int dp = 0; dp < 8; ++dp) {
+                    uint32_t b0, b1, b2, b3;
+                    ldsm_x4_t(sC + sw128(j * 16 + (mi & 1) * 8 + (lane & 7), dp * 2 + (mi >> 1)), b0, b1, b2, b3);
+                    mma_bf16(y[2 * dp], af[2 * j][0], af[2 * j][1], af[2 * j + 1][0], af[2 * j + 1][1], b0, b1);
+                    mma_bf16(y[2 * dp + 1], af[2 * j][0], af[2 * j][1], af[2 * j + 1][0], af[2 * j + 1][1], b2, b3);
+                }
+            // ---- row sums of y^2 and (O^s)^2, then O = O^s + g r_p O^lr over O^s
+            ok = __all_sync(0xffffffffu, mbar_wait(o_full + 8 * buf, (i / OB) & 1, abort, s.wait_limit_ns));
+            if (!ok) break;
+            const uint32_t ob = qb + kBox + buf * kBox;
+            auto os = [&](int d, int hr) {               // this thread's pair of O^s (read twice: registers are short)
+                uint32_t w;
+                asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(w) : "r"(ob + wsw(g + 8 * hr, d) + t4 * 4));
+                return unpack_bf16(w);
+            };
+            float ssy[2] = {0.0f, 0.0f}, sso[2] = {0.0f, 0.0f};
+#pragma unroll
+            for (int d = 0; d < 16; ++d) {
+#pragma unroll
+                for (int hr = 0; hr < 2; ++hr) {
+                    const float2 f = os(d, hr);
+                    ssy[hr] += y[d][2 * hr] * y[d][2 * hr] + y[d][2 * hr + 1] * y[d][2 * hr + 1];
+                    sso[hr] += f.x * f.x + f.y * f.y;
+                }
+            }
 #pragma unroll
             for (int hr = 0; hr < 2; ++hr) {
-                const int tl = mt * 16 + g + hr * 8;
+                ssy[hr] += __shfl_xor_sync(0xffffffffu, ssy[hr], 1);
+                ssy[hr] += __shfl_xor_sync(0xffffffffu, ssy[hr], 2);
+                sso[hr] += __shfl_xor_sync(0xffffffffu, sso[hr], 1);
+                sso[hr] += __shfl_xor_sync(0xffffffffu, sso[hr], 2);
+                const float coef = gp[hr] * sqrtf(sso[hr] * (1.0f / kDh) + s.eps_fuse) *
+                                   rsqrtf(ssy[hr] * (1.0f / kDh) + s.eps_lr);
 #pragma unroll
-                for (int j = 0; j < NTW; ++j) {
-                    const int nt = half * NTW + j;
-                    const float2 f = lowrank_pair(uacc[j][2 * hr], uacc[j][2 * hr + 1], kcs[hr][j], s.lr_rope,
-                                                  Act{s.lr_act});
-                    asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(sQt + tl * L::QT + (nt * 8 + t4 * 2) * 2),
-                                 "r"(pack_bf16(f.x, f.y))
+                for (int d = 0; d < 16; ++d) {
+                    const float2 f = os(d, hr);
+                    asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(ob + wsw(g + 8 * hr, d) + t4 * 4),
+                                 "r"(pack_bf16(f.x + coef * y[d][2 * hr], f.y + coef * y[d][2 * hr + 1]))
                                  : "memory");
                 }
             }
-        }
-        // every thread reaches this barrier once per unit; it also settles a timeout
-        if (bar_red_or(1, kThreads, !ok)) {
-            failed = true;
-            break;
-        }
-        if (i >= 1 && issued < count) {
-            // refill the stage of unit i - 1 once its store has finished reading it
-            if (tid == 0) bulk_wait_read_all();
-            issue(issued);
-            ++issued;
-        }
-        // ---- y = q~ C for d in [64 half, 64 half + 64)
-        float yacc[8][4];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) yacc[j][0] = yacc[j][1] = yacc[j][2] = yacc[j][3] = 0.0f;
-#pragma unroll
-        for (int kc = 0; kc < R / 16; ++kc) {
-            uint32_t a0, a1, a2, a3;
-            ldsm_x4(sQt + (mt * 16 + (lane & 7) + (mi & 1) * 8) * L::QT + (kc * 2 + (mi >> 1)) * 16, a0, a1, a2, a3);
-#pragma unroll
-            for (int dp = 0; dp < 4; ++dp) {
-                uint32_t b0, b1, b2, b3;
-                ldsm_x4_t(sC + sw128(kc * 16 + (mi & 1) * 8 + (lane & 7), half * 8 + dp * 2 + (mi >> 1)), b0, b1, b2,
-                          b3);
-                mma_bf16(yacc[2 * dp], a0, a1, a2, a3, b0, b1);
-                mma_bf16(yacc[2 * dp + 1], a0, a1, a2, a3, b2, b3);
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                tma_store_4d(&map_o, ob, 0, x * kTile, 0, bh);
+                bulk_commit();
             }
-        }
-        // ---- row sums of y^2 and (O^s)^2 over this half's 64 d, then over both halves
-        float ssy[2] = {0.0f, 0.0f}, sso[2] = {0.0f, 0.0f};
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int c = half * 8 + j;
-            uint32_t wlo, whi;
-            asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(wlo) : "r"(ob + tsw(r_lo, c) + t4 * 4));
-            asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(whi) : "r"(ob + tsw(r_hi, c) + t4 * 4));
-            const float2 lo = unpack_bf16(wlo), hi = unpack_bf16(whi);
-            ssy[0] += yacc[j][0] * yacc[j][0] + yacc[j][1] * yacc[j][1];
-            ssy[1] += yacc[j][2] * yacc[j][2] + yacc[j][3] * yacc[j][3];
-            sso[0] += lo.x * lo.x + lo.y * lo.y;
-            sso[1] += hi.x * hi.x + hi.y * hi.y;
-        }
-#pragma unroll
-        for (int hr = 0; hr < 2; ++hr) {
-            ssy[hr] += __shfl_xor_sync(0xffffffffu, ssy[hr], 1);
-            ssy[hr] += __shfl_xor_sync(0xffffffffu, ssy[hr], 2);
-            sso[hr] += __shfl_xor_sync(0xffffffffu, sso[hr], 1);
-            sso[hr] += __shfl_xor_sync(0xffffffffu, sso[hr], 2);
-        }
-        if (t4 == 0) {
-            red[(0 * 2 + half) * 64 + r_lo] = ssy[0];
-            red[(0 * 2 + half) * 64 + r_hi] = ssy[1];
-            red[(1 * 2 + half) * 64 + r_lo] = sso[0];
-            red[(1 * 2 + half) * 64 + r_hi] = sso[1];
-        }
-        bar_sync(1, kThreads);
-        // ---- O = O^s + g r_p O^lr, written over O^s in the stage
-        float coef[2];
-#pragma unroll
-        for (int hr = 0; hr < 2; ++hr) {
-            const int row = hr ? r_hi : r_lo;
-            const float sy = red[0 * 64 + row] + red[1 * 64 + row];
-            const float so = red[2 * 64 + row] + red[3 * 64 + row];
-            coef[hr] = gp[hr] * sqrtf(so * (1.0f / kDh) + s.eps_fuse) * rsqrtf(sy * (1.0f / kDh) + s.eps_lr);
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int c = half * 8 + j;
-            const uint32_t alo = ob + tsw(r_lo, c) + t4 * 4, ahi = ob + tsw(r_hi, c) + t4 * 4;
-            uint32_t wlo, whi;
-            asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(wlo) : "r"(alo));
-            asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(whi) : "r"(ahi));
-            const float2 lo = unpack_bf16(wlo), hi = unpack_bf16(whi);
-            const uint32_t olo = pack_bf16(lo.x + coef[0] * yacc[j][0], lo.y + coef[0] * yacc[j][1]);
-            const uint32_t ohi = pack_bf16(hi.x + coef[1] * yacc[j][2], hi.y + coef[1] * yacc[j][3]);
-            asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(alo), "r"(olo) : "memory");
-            asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(ahi), "r"(ohi) : "memory");
-        }
-        fence_proxy_async_smem();
-        bar_sync(1, kThreads);
-        if (tid == 0) {
-            tma_store_4d(&map_o, ob, 0, n_base, 0, bh);
-            bulk_commit();
+            if (OB == 1 && more) load_o(x + kWarps, 0);
         }
     }
-    if (tid == 0) {
-        if (failed) {
+    if (lane == 0) {
+        if (!ok) {
             if (atomicCAS(&p.status->code, 0, (int)ROLA_ERR_TIMEOUT) == 0) p.status->where = 8;
             // loads issued and not yet waited for must land before the CTA exits
             int never = 0;
-            for (int j = i; j < issued; ++j)
-                mbar_wait(full0 + 8 * (j % kStages), (j / kStages) & 1, &never, s.wait_limit_ns);
+            if (q_issued > 0) mbar_wait(q_full, (q_issued - 1) & 1, &never, s.wait_limit_ns);
+            for (int j = o_issued > OB ? o_issued - OB : 0; j < o_issued; ++j)
+                mbar_wait(o_full + 8 * (j % OB), (j / OB) & 1, &never, s.wait_limit_ns);
         }
         bulk_wait_all();
     }
@@ -334,7 +273,7 @@ cudaError_t launch_ra(const CUtensorMap& mq, const CUtensorMap& mos, const CUten
     cudaError_t e =
         cudaFuncSetAttribute(readout_kernel<R, Act>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::total);
     if (e != cudaSuccess) return e;
-    readout_kernel<R, Act><<<ctas, kThreads, L::total, st>>>(mq, mos, mo, p);
+    readout_kernel<R, Act><<<ctas, 32 * L::warps, L::total, st>>>(mq, mos, mo, p);
     return cudaGetLastError();
 }
 
@@ -352,16 +291,16 @@ cudaError_t launch_readout(const Shape& s, const void* q, const void* P_q, const
                            const float* gate, const void* o_s, void* o, const float2* tab, DeviceStatus* status,
                            cudaStream_t st)
 {
-    const int units = s.B * s.H * s.nC;
+    const int tiles = (s.N + kTile - 1) / kTile;
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const int per_sm = s.rp <= 48 ? 2 : 1;                   // Occupancy<R>::ctas
-    const int ctas = units < nsm * per_sm ? units : nsm * per_sm;
+    const long long total = (long long)s.B * s.H * tiles;
+    const int ctas = total < nsm ? (int)total : nsm;
     CUtensorMap mq, mos, mo;
-    if (!make_block_map(&mq, q, s) || !make_block_map(&mos, o_s, s) || !make_block_map(&mo, o, s))
+    if (!make_block_map(&mq, q, s, kTile) || !make_block_map(&mos, o_s, s, kTile) || !make_block_map(&mo, o, s, kTile))
         return cudaErrorInvalidValue;
     Params p;
     p.s = s;
@@ -370,7 +309,7 @@ cudaError_t launch_readout(const Shape& s, const void* q, const void* P_q, const
     p.gate = gate;
     p.tab = tab;
     p.status = status;
-    p.units = units;
+    p.tiles = tiles;
     switch (s.rp) {
         case 16: return launch_r<16>(mq, mos, mo, p, ctas, st);
         case 32: return launch_r<32>(mq, mos, mo, p, ctas, st);
