@@ -200,12 +200,15 @@ rola_status_t run_summary(const rola_config_t& c, const Shape& s, const Workspac
     return ROLA_OK;
 }
 
-// q^r, k^r and the block means; v in block order too when v is given and the geometry is cubes.
+// q^r, k^r (with `rows`) and the block means (with `means`); v in block order too when v is given and the
+// geometry is cubes.
 cudaError_t rope_pool(const rola_config_t& c, const Shape& s, const Workspace& w, const void* q, const void* k,
-                      const void* v, void* ws, cudaStream_t st)
+                      const void* v, bool rows, bool means, void* ws, cudaStream_t st)
 {
-    return launch_rope_pool(c, s, q, k, s.cube ? v : nullptr, at<float2>(ws, w.table), at<void>(ws, w.qr),
-                            at<void>(ws, w.kr), at<void>(ws, w.vp), at<float>(ws, w.qbar), at<float>(ws, w.kbar), st);
+    return launch_rope_pool(c, s, q, k, s.cube ? v : nullptr, at<float2>(ws, w.table),
+                            rows ? at<void>(ws, w.qr) : nullptr, rows ? at<void>(ws, w.kr) : nullptr,
+                            at<void>(ws, w.vp), means ? at<float>(ws, w.qbar) : nullptr,
+                            means ? at<float>(ws, w.kbar) : nullptr, st);
 }
 
 // The v rows the sparse kernels read: the caller's v, or its block-ordered copy in cube geometry.
@@ -227,9 +230,9 @@ cudaError_t select_blocks(const Shape& s, const Workspace& w, int32_t* kv_idx, v
 }
 
 rola_status_t run_mask(const rola_config_t& c, const Shape& s, const Workspace& w, const void* q, const void* k,
-                       const void* v, int32_t* kv_idx, void* ws, cudaStream_t st)
+                       const void* v, bool rows, int32_t* kv_idx, void* ws, cudaStream_t st)
 {
-    ROLA_TRY(rope_pool(c, s, w, q, k, v, ws, st));
+    ROLA_TRY(rope_pool(c, s, w, q, k, v, rows, true, ws, st));
     ROLA_TRY(select_blocks(s, w, kv_idx, ws, st));
     return ROLA_OK;
 }
@@ -237,7 +240,7 @@ rola_status_t run_mask(const rola_config_t& c, const Shape& s, const Workspace& 
 // Backward workspace: the status word and RoPE table as in the forward
 // workspace, the rotated copies, fp32 gradient rows and partials.
 struct BwdWorkspace {
-    size_t status, table, qr, kr, vp, qbar, kbar, dOs, Dv, dq, dk, dv, dg, partC, partPq, partPk, dC, tr_off, tr_list,
+    size_t status, table, qr, kr, vp, dOs, Dv, dq, dk, dv, dg, partC, partPq, partPk, dC, tr_off, tr_list,
         dOs_b, lse_b, Dv_b, total;
 };
 
@@ -255,8 +258,6 @@ BwdWorkspace bwd_layout(const rola_config_t& c)
     w.qr = off; off = align_up(off + esz * brows * kDh);
     w.kr = off; off = align_up(off + esz * brows * kDh);
     w.vp = off; off = align_up(off + cube * esz * brows * kDh);
-    w.qbar = off; off = align_up(off + 4 * bh * s.nB * kDh);
-    w.kbar = off; off = align_up(off + 4 * bh * s.nB * kDh);
     w.dOs = off; off = align_up(off + esz * rows * kDh);
     w.Dv = off; off = align_up(off + 4 * rows);
     w.dq = off; off = align_up(off + 4 * rows * kDh);
@@ -307,7 +308,7 @@ rola_status_t forward_impl(const rola_config_t* cfg, const void* q, const void* 
         // stage 2: block scores + top-k, and the summary combine
         const int ctas = prepass_ctas(s, kMaxPrepassCtas);
         if (ctas <= 0) return ROLA_ERR_CUDA;
-        ROLA_TRY(rope_pool(*cfg, s, w, q, k, v, ws, st));
+        ROLA_TRY(rope_pool(*cfg, s, w, q, k, v, true, true, ws, st));
         ROLA_TRY(launch_prepass(s, ctas, nullptr, k, v, P_k, at<float2>(ws, w.table), nullptr, nullptr, nullptr,
                                 nullptr, at<float>(ws, w.partials), at<DeviceStatus>(ws, w.status), st));
         ROLA_TRY(mark(1));
@@ -328,7 +329,7 @@ rola_status_t forward_impl(const rola_config_t* cfg, const void* q, const void* 
                                         at<__nv_bfloat16>(ws, w.Cbf), st));
     } else {
         // stage 1: the block mask; stage 2: the summary
-        ROLA_CHECK(run_mask(*cfg, s, w, q, k, v, kv, ws, st));
+        ROLA_CHECK(run_mask(*cfg, s, w, q, k, v, true, kv, ws, st));
         ROLA_TRY(mark(1));
         ROLA_CHECK(run_summary(*cfg, s, w, k, v, P_k, at<float>(ws, w.C), at<float>(ws, w.z),
                                at<__nv_bfloat16>(ws, w.Cbf), ws, st));
@@ -427,7 +428,7 @@ rola_status_t rola_block_mask(const rola_config_t* cfg, const void* q, const voi
     Workspace w = layout(*cfg);
     Shape s = make_shape(*cfg);
     ROLA_CHECK(prologue(*cfg, ws, w, st));
-    return run_mask(*cfg, s, w, q, k, nullptr, kv_idx, ws, st);
+    return run_mask(*cfg, s, w, q, k, nullptr, false, kv_idx, ws, st);
 }
 
 rola_status_t rola_sparse_attn(const rola_config_t* cfg, const void* q, const void* k, const void* v,
@@ -442,8 +443,8 @@ rola_status_t rola_sparse_attn(const rola_config_t* cfg, const void* q, const vo
     Workspace w = layout(*cfg);
     Shape s = make_shape(*cfg);
     ROLA_CHECK(prologue(*cfg, ws, w, st));
-    // rotated copies in block order (the pooled means are a by-product here)
-    ROLA_TRY(rope_pool(*cfg, s, w, q, k, v, ws, st));
+    // rotated copies in block order
+    ROLA_TRY(rope_pool(*cfg, s, w, q, k, v, true, false, ws, st));
     ROLA_TRY(launch_sparse_attn(cfg->dtype, s, at<void>(ws, w.qr), at<void>(ws, w.kr), sparse_v(s, w, v, ws), kv_idx,
                                 o_s, nullptr, at<DeviceStatus>(ws, w.status), st));
     return ROLA_OK;
@@ -533,8 +534,7 @@ rola_status_t rola_backward(const rola_config_t* cfg, const void* q, const void*
     ROLA_TRY(cudaMemsetAsync(at<uint8_t>(ws, w.status), 0, sizeof(DeviceStatus), st));
     ROLA_TRY(launch_rope_table(*cfg, at<float2>(ws, w.table), st));
     ROLA_TRY(launch_rope_pool(*cfg, s, q, k, s.cube ? v : nullptr, at<float2>(ws, w.table), at<void>(ws, w.qr),
-                              at<void>(ws, w.kr), s.cube ? at<void>(ws, w.vp) : nullptr, at<float>(ws, w.qbar),
-                              at<float>(ws, w.kbar), st));
+                              at<void>(ws, w.kr), s.cube ? at<void>(ws, w.vp) : nullptr, nullptr, nullptr, st));
     BackwardArgs a;
     a.q = q; a.k = k; a.v = v; a.P_q = P_q; a.P_k = P_k; a.o_s = o_s; a.dO = dO;
     a.C = C; a.gate = gate; a.lse = lse; a.kv_idx = kv_idx;

@@ -42,205 +42,157 @@ cudaError_t launch_rope_table(const rola_config_t& cfg, float2* tab, cudaStream_
 }
 
 // ---------------------------------------------------------------------------
-// rotate + pool: one CTA per (64-token block, head, q|k).  256 threads: 16 per
-// token row (8 coordinates = 4 pairs each), 16 rows per pass, 4 passes.  Writes
-// the rotated rows in the storage dtype and the fp32 block mean of the
+// rotate + pool: one CTA per (64-slot block, head, q | k | v).  Eight warps: warp w
+// takes slots 8 w .. 8 w + 7, a lane four coordinates (two pairs), so a token's grid
+// position is the same for the whole warp.  Writes the rotated rows in the storage
+// dtype (unless the caller only wants the mask) and the fp32 block mean of the
 // fp32-rotated (unrounded) values.  The block mean is the pairwise sum of the
-// block's 64 slots in slot order (slots past the sequence hold +0), divided
-// once by the token count: the evaluation order the block mask is defined
-// with, so that every kernel computing it gives the same bits.
+// block's 64 slots in slot order (empty slots hold +0), divided once by the token
+// count: the evaluation order the block mask is defined with, so that every kernel
+// computing it gives the same bits.  A lane adds its warp's eight slots (tree
+// levels 1 to 3) in registers; the 8 nodes per coordinate pass through shared memory.
+//
+// Cube geometry: slots 8 w .. are two runs of four tokens along a grid row.  The
+// rotated rows are written in block order (row 64 b + slot of the head's Np rows,
+// zeros for slots outside the grid, so that the sparse kernels read finite values
+// there); z = 2 copies v into the same order.
+//
+// HBM wants 512 B read (and 512 B written) per token of q and k at 16 bits.  With
+// 16 lanes a token and each lane's position and table rows computed on its own, a
+// thread took 550-670 instructions for its 32 values and issue was the bound.
+// 720p layer (40 heads, 75600 tokens): means alone 380 us (4.1 TB/s read; they used
+// to come with the rows, 771 us for both); 480p cubes of q, k and v 522 -> 348 us.
 
-// Pairwise sum of the 64 values col[0], col[stride], ..., col[63 stride]:
-// sum(x[0..n)) = sum(x[0..n/2)) + sum(x[n/2..n)), evaluated level by level.
-__device__ __forceinline__ float pairwise64(const float* col, int stride)
-{
-    float v[kBlock];
-#pragma unroll
-    for (int i = 0; i < kBlock; ++i) v[i] = col[i * stride];
-#pragma unroll
-    for (int w = 1; w < kBlock; w *= 2)
-#pragma unroll
-        for (int i = 0; i < kBlock; i += 2 * w) v[i] = v[i] + v[i + w];
-    return v[0];
-}
-
+// Four coordinates of a row.
 template <typename T>
-struct Vec8;
+struct Vec4;
 template <>
-struct Vec8<__nv_bfloat16> {
-    __device__ static void load(const __nv_bfloat16* p, float (&x)[8])
+struct Vec4<__nv_bfloat16> {
+    using Raw = uint2;
+    __device__ static void unpack(const Raw& r, float (&x)[4])
     {
-        uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
-        uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float2 f = unpack_bf16(w[i]);
-            x[2 * i] = f.x;
-            x[2 * i + 1] = f.y;
-        }
+        const float2 a = unpack_bf16(r.x), b = unpack_bf16(r.y);
+        x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
     }
-    __device__ static void store(__nv_bfloat16* p, const float (&x)[8])
-    {
-        uint4 u = make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]),
-                             pack_bf16(x[6], x[7]));
-        *reinterpret_cast<uint4*>(p) = u;
-    }
+    __device__ static Raw pack(const float (&x)[4]) { return make_uint2(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3])); }
+    __device__ static Raw zero() { return make_uint2(0u, 0u); }
 };
 template <>
-struct Vec8<float> {
-    __device__ static void load(const float* p, float (&x)[8])
-    {
-        float4 a = __ldg(reinterpret_cast<const float4*>(p));
-        float4 b = __ldg(reinterpret_cast<const float4*>(p) + 1);
-        x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
-        x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
-    }
-    __device__ static void store(float* p, const float (&x)[8])
-    {
-        reinterpret_cast<float4*>(p)[0] = make_float4(x[0], x[1], x[2], x[3]);
-        reinterpret_cast<float4*>(p)[1] = make_float4(x[4], x[5], x[6], x[7]);
-    }
+struct Vec4<float> {
+    using Raw = float4;
+    __device__ static void unpack(const Raw& r, float (&x)[4]) { x[0] = r.x; x[1] = r.y; x[2] = r.z; x[3] = r.w; }
+    __device__ static Raw pack(const float (&x)[4]) { return make_float4(x[0], x[1], x[2], x[3]); }
+    __device__ static Raw zero() { return make_float4(0.0f, 0.0f, 0.0f, 0.0f); }
 };
 
-template <typename T>
+template <typename T, bool kCube>
 __global__ void __launch_bounds__(256) rope_pool_kernel(Shape s, const T* __restrict__ q, const T* __restrict__ k,
-                                                        const float2* __restrict__ tab, T* __restrict__ qr,
-                                                        T* __restrict__ kr, float* __restrict__ qbar,
-                                                        float* __restrict__ kbar)
+                                                        const T* __restrict__ v, const float2* __restrict__ tab,
+                                                        T* __restrict__ qr, T* __restrict__ kr, T* __restrict__ vp,
+                                                        float* __restrict__ qbar, float* __restrict__ kbar)
 {
-    __shared__ __align__(16) float rot[kBlock][kDh];      // fp32 rotated rows, slot order
-    const int blk = blockIdx.x, bh = blockIdx.y;
-    const T* x = blockIdx.z == 0 ? q : k;
-    T* xr = blockIdx.z == 0 ? qr : kr;
-    float* xbar = blockIdx.z == 0 ? qbar : kbar;
-    const int c8 = threadIdx.x & 15;        // coordinates 8*c8 .. 8*c8+7 (pairs 4*c8 .. 4*c8+3)
-    const int rsub = threadIdx.x >> 4;      // row within a pass; rows rsub + 16 * pass
-    const int n0 = blk * kBlock + rsub;
-    constexpr int kPasses = kBlock / 16;
-    // all loads first: four 16- or 32-byte vectors in flight per thread
-    float v[kPasses][8];
-#pragma unroll
-    for (int pass = 0; pass < kPasses; ++pass) {
-        const int n = n0 + 16 * pass;
-        if (n < s.N) Vec8<T>::load(x + ((size_t)bh * s.N + n) * kDh + c8 * 8, v[pass]);
-    }
-    // grid position of the first row, then advanced by 16 tokens per pass
-    const int hw = s.Hh * s.Ww;
-    int t = n0 / hw, rem = n0 - t * hw;
-    int xx = rem / s.Ww, yy = rem - xx * s.Ww;
-    // table row base of each of this thread's 4 pairs: the pair's axis is fixed
-    int axis[4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        const int m = c8 * 4 + p;
-        axis[p] = m < s.pt ? 0 : (m < s.pt + s.px ? 1 : 2);
-    }
-#pragma unroll
-    for (int pass = 0; pass < kPasses; ++pass) {
-        const int n = n0 + 16 * pass;
-        float o[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        if (n < s.N) {
-#pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                const int row = axis[p] == 0 ? t : (axis[p] == 1 ? s.T + xx : s.T + s.Hh + yy);
-                const float2 cs = __ldg(tab + row * kPairs + c8 * 4 + p);
-                const float2 y = rope_rotate(v[pass][2 * p], v[pass][2 * p + 1], cs);
-                o[2 * p] = y.x;
-                o[2 * p + 1] = y.y;
-            }
-            Vec8<T>::store(xr + ((size_t)bh * s.N + n) * kDh + c8 * 8, o);
-        }
-        float4* dst = reinterpret_cast<float4*>(&rot[rsub + 16 * pass][c8 * 8]);
-        dst[0] = make_float4(o[0], o[1], o[2], o[3]);
-        dst[1] = make_float4(o[4], o[5], o[6], o[7]);
-        yy += 16;                           // advance to the token 16 further on
-        while (yy >= s.Ww) {
-            yy -= s.Ww;
-            if (++xx == s.Hh) {
-                xx = 0;
-                ++t;
-            }
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x < kDh) {
-        const int cnt = min(kBlock, s.N - blk * kBlock);
-        const float sum = pairwise64(&rot[0][threadIdx.x], kDh);
-        // with 128-token query blocks the query side keeps the sum (the 128-token tree's left or right half)
-        xbar[((size_t)bh * s.nB + blk) * kDh + threadIdx.x] = (blockIdx.z == 0 && s.qb2) ? sum : sum / (float)cnt;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// The same pass in cube geometry: one CTA per (cube, head, q|k|v).  Thread
-// (rsub, c8) handles slot rsub + 16 dt of the cube for dt = 0..3, i.e. grid
-// position (t0 + dt, x0 + rsub / 4, y0 + rsub % 4).  The rotated rows are
-// written in block order (row 64 b + slot of the head's Np rows, zeros for
-// slots outside the grid, so that the sparse kernels read finite values
-// there); the v slice copies v into the same order without rotating it.
-
-template <typename T>
-__global__ void __launch_bounds__(256) rope_pool_cube_kernel(Shape s, const T* __restrict__ q,
-                                                             const T* __restrict__ k, const T* __restrict__ v,
-                                                             const float2* __restrict__ tab, T* __restrict__ qr,
-                                                             T* __restrict__ kr, T* __restrict__ vp,
-                                                             float* __restrict__ qbar, float* __restrict__ kbar)
-{
-    __shared__ __align__(16) float rot[kBlock][kDh];      // fp32 rotated rows, slot order
+    using Raw = typename Vec4<T>::Raw;
+    __shared__ __align__(16) float nodes[8][kDh];            // level-3 nodes of the pairwise sum, slot order
     const int blk = blockIdx.x, bh = blockIdx.y, z = blockIdx.z;
     const T* x = z == 0 ? q : (z == 1 ? k : v);
-    T* xr = z == 0 ? qr : (z == 1 ? kr : vp);
-    const int c8 = threadIdx.x & 15;
-    const int rsub = threadIdx.x >> 4;
-    constexpr int kPasses = kBlock / 16;
-    const CubeOrigin o = cube_origin(s, blk);
-    float v8[kPasses][8];
+    T* xr = z == 0 ? qr : (z == 1 ? kr : vp);                // null: the rows are not wanted
+    float* xbar = z == 0 ? qbar : (z == 1 ? kbar : nullptr);   // null: the means are not wanted
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (warp-uniform)
+    // first token of each run (chunks: one run of eight, cubes: two of four) and how many tokens it holds
+    constexpr int kRuns = kCube ? 2 : 1, kLen = 8 / kRuns;
+    int n0[kRuns], cnt[kRuns], t, xx, yy, tokens;
+    if constexpr (kCube) {
+        const CubeOrigin o = cube_origin(s, blk);
+        t = o.t + (warp >> 1);
+        xx = o.x + 2 * (warp & 1);
+        yy = o.y;
 #pragma unroll
-    for (int dt = 0; dt < kPasses; ++dt) {
-        const int n = cube_token(s, o, rsub + 16 * dt);
-        if (n >= 0) Vec8<T>::load(x + ((size_t)bh * s.N + n) * kDh + c8 * 8, v8[dt]);
+        for (int r = 0; r < 2; ++r) {
+            n0[r] = (t * s.Hh + xx + r) * s.Ww + yy;
+            cnt[r] = t < s.T && xx + r < s.Hh ? min(4, s.Ww - yy) : 0;
+        }
+        tokens = min(4, s.T - o.t) * min(4, s.Hh - o.x) * min(4, s.Ww - o.y);
+    } else {
+        n0[0] = blk * kBlock + 8 * warp;
+        cnt[0] = min(8, max(0, s.N - n0[0]));
+        const int hw = s.Hh * s.Ww;
+        t = n0[0] / hw;
+        const int rem = n0[0] - t * hw;
+        xx = rem / s.Ww;
+        yy = rem - xx * s.Ww;
+        tokens = min(kBlock, s.N - blk * kBlock);
     }
-    int axis[4];
+    // all loads first: eight 8- or 16-byte vectors in flight per thread
+    Raw raw[8];
+    const Raw* src = reinterpret_cast<const Raw*>(x + (size_t)bh * s.N * kDh) + lane;
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        const int m = c8 * 4 + p;
-        axis[p] = m < s.pt ? 0 : (m < s.pt + s.px ? 1 : 2);
+    for (int j = 0; j < 8; ++j) {
+        const int r = j / kLen, i = j % kLen;
+        raw[j] = i < cnt[r] ? __ldg(src + (size_t)(n0[r] + i) * 32) : Vec4<T>::zero();
     }
-    const int xx = o.x + (rsub >> 2), yy = o.y + (rsub & 3);
+    // chunks: Np = N and a slot past the sequence has no row; cubes: every slot has one
+    Raw* dst = xr ? reinterpret_cast<Raw*>(xr + ((size_t)bh * s.Np + (size_t)blk * kBlock + 8 * warp) * kDh) + lane : nullptr;
+    if (z == 2) {
 #pragma unroll
-    for (int dt = 0; dt < kPasses; ++dt) {
-        const int slot = rsub + 16 * dt;
-        const int n = cube_token(s, o, slot);
-        float out[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        if (n >= 0) {
-            if (z == 2) {
+        for (int j = 0; j < 8; ++j) dst[j * 32] = raw[j];
+        return;
+    }
+    // (cos, sin) of this lane's two pairs; from token to token along a grid row only the column's pairs change
+    const int m = 2 * lane;
+    const int ax0 = m < s.pt ? 0 : (m < s.pt + s.px ? 1 : 2), ax1 = m + 1 < s.pt ? 0 : (m + 1 < s.pt + s.px ? 1 : 2);
+    const float2 *p0, *p1;
+    float2 c0, c1;
+    auto seek = [&]() {
+        p0 = tab + (ax0 == 0 ? t : (ax0 == 1 ? s.T + xx : s.T + s.Hh + yy)) * kPairs + m;
+        p1 = tab + (ax1 == 0 ? t : (ax1 == 1 ? s.T + xx : s.T + s.Hh + yy)) * kPairs + m + 1;
+        c0 = __ldg(p0);
+        c1 = __ldg(p1);
+    };
+    float sum[4];
+    float y[8][4];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) out[i] = v8[dt][i];
+    for (int j = 0; j < 8; ++j) {
+        const int r = j / kLen, i = j % kLen;
+        if (i < cnt[r]) {
+            if (i == 0) {
+                if (r > 0) ++xx;
+                seek();
             } else {
-                const int t = o.t + dt;
-#pragma unroll
-                for (int p = 0; p < 4; ++p) {
-                    const int row = axis[p] == 0 ? t : (axis[p] == 1 ? s.T + xx : s.T + s.Hh + yy);
-                    const float2 cs = __ldg(tab + row * kPairs + c8 * 4 + p);
-                    const float2 y = rope_rotate(v8[dt][2 * p], v8[dt][2 * p + 1], cs);
-                    out[2 * p] = y.x;
-                    out[2 * p + 1] = y.y;
+                if (++yy < s.Ww) {
+                    if (ax0 == 2) c0 = __ldg(p0 += kPairs);
+                    if (ax1 == 2) c1 = __ldg(p1 += kPairs);
+                } else {
+                    yy = 0;
+                    if (++xx == s.Hh) {
+                        xx = 0;
+                        ++t;
+                    }
+                    seek();
                 }
             }
+            float w[4];
+            Vec4<T>::unpack(raw[j], w);
+            const float2 a = rope_rotate(w[0], w[1], c0), b = rope_rotate(w[2], w[3], c1);
+            y[j][0] = a.x; y[j][1] = a.y; y[j][2] = b.x; y[j][3] = b.y;
+        } else {
+            y[j][0] = y[j][1] = y[j][2] = y[j][3] = 0.0f;    // an empty slot of the pairwise sum
         }
-        Vec8<T>::store(xr + ((size_t)bh * s.Np + (size_t)blk * kBlock + slot) * kDh + c8 * 8, out);
-        if (z != 2) {
-            float4* dst = reinterpret_cast<float4*>(&rot[slot][c8 * 8]);
-            dst[0] = make_float4(out[0], out[1], out[2], out[3]);
-            dst[1] = make_float4(out[4], out[5], out[6], out[7]);
-        }
+        if constexpr (kCube)
+            if (i == kLen - 1 && r == 0 && cnt[0] > 0) yy -= cnt[0] - 1;   // back to the run's first column
+        if (dst && (kCube || i < cnt[r])) dst[j * 32] = Vec4<T>::pack(y[j]);
     }
-    if (z == 2) return;
+    if (!xbar) return;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        sum[i] = ((y[0][i] + y[1][i]) + (y[2][i] + y[3][i])) + ((y[4][i] + y[5][i]) + (y[6][i] + y[7][i]));
+    *reinterpret_cast<float4*>(&nodes[warp][4 * lane]) = make_float4(sum[0], sum[1], sum[2], sum[3]);
     __syncthreads();
     if (threadIdx.x < kDh) {
-        const int cnt = min(4, s.T - o.t) * min(4, s.Hh - o.x) * min(4, s.Ww - o.y);
-        (z == 0 ? qbar : kbar)[((size_t)bh * s.nB + blk) * kDh + threadIdx.x] =
-            pairwise64(&rot[0][threadIdx.x], kDh) / (float)cnt;
+        const int c = threadIdx.x;
+        const float all = ((nodes[0][c] + nodes[1][c]) + (nodes[2][c] + nodes[3][c])) +
+                          ((nodes[4][c] + nodes[5][c]) + (nodes[6][c] + nodes[7][c]));
+        // with 128-token query blocks the query side keeps the sum (the 128-token tree's left or right half)
+        xbar[((size_t)bh * s.nB + blk) * kDh + c] = z == 0 && s.qb2 ? all : all / (float)tokens;
     }
 }
 
@@ -248,14 +200,9 @@ template <typename T>
 cudaError_t launch_rope_pool_t(const Shape& s, const void* q, const void* k, const void* v, const float2* tab,
                                void* qr, void* kr, void* vp, float* qbar, float* kbar, cudaStream_t st)
 {
-    if (s.cube) {
-        dim3 grid(s.nB, s.B * s.H, v ? 3 : 2);
-        rope_pool_cube_kernel<T><<<grid, 256, 0, st>>>(s, (const T*)q, (const T*)k, (const T*)v, tab, (T*)qr,
-                                                       (T*)kr, (T*)vp, qbar, kbar);
-    } else {
-        dim3 grid(s.nB, s.B * s.H, 2);
-        rope_pool_kernel<T><<<grid, 256, 0, st>>>(s, (const T*)q, (const T*)k, tab, (T*)qr, (T*)kr, qbar, kbar);
-    }
+    const dim3 grid(s.nB, s.B * s.H, s.cube && v ? 3 : 2);
+    auto kernel = s.cube ? rope_pool_kernel<T, true> : rope_pool_kernel<T, false>;
+    kernel<<<grid, 256, 0, st>>>(s, (const T*)q, (const T*)k, (const T*)v, tab, (T*)qr, (T*)kr, (T*)vp, qbar, kbar);
     return cudaGetLastError();
 }
 
