@@ -178,8 +178,7 @@ rola_status_t check_ws(const rola_config_t& c, const void* ws, size_t ws_bytes)
 // Start of every entry point: clear the status word, build the RoPE table.
 rola_status_t prologue(const rola_config_t& c, void* ws, const Workspace& w, cudaStream_t st)
 {
-    ROLA_TRY(cudaMemsetAsync(at<uint8_t>(ws, w.status), 0, sizeof(DeviceStatus), st));
-    ROLA_TRY(launch_rope_table(c, at<float2>(ws, w.table), st));
+    ROLA_TRY(launch_rope_table(c, at<float2>(ws, w.table), at<DeviceStatus>(ws, w.status), st));
     return ROLA_OK;
 }
 
@@ -531,8 +530,7 @@ rola_status_t rola_backward(const rola_config_t* cfg, const void* q, const void*
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) || ws_bytes < w.total) return ROLA_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const Shape s = make_shape(*cfg);
-    ROLA_TRY(cudaMemsetAsync(at<uint8_t>(ws, w.status), 0, sizeof(DeviceStatus), st));
-    ROLA_TRY(launch_rope_table(*cfg, at<float2>(ws, w.table), st));
+    ROLA_TRY(launch_rope_table(*cfg, at<float2>(ws, w.table), at<DeviceStatus>(ws, w.status), st));
     ROLA_TRY(launch_rope_pool(*cfg, s, q, k, s.cube ? v : nullptr, at<float2>(ws, w.table), at<void>(ws, w.qr),
                               at<void>(ws, w.kr), s.cube ? at<void>(ws, w.vp) : nullptr, nullptr, nullptr, st));
     BackwardArgs a;

@@ -208,6 +208,7 @@ __global__ void __launch_bounds__(kBT) lr_bwd_q_kernel(Shape s, const T* __restr
                                                        float* __restrict__ dg_h, float* __restrict__ partC,
                                                        float* __restrict__ partPq)
 {
+    chain_begin();
     extern __shared__ float lsm[];
     const LrSmem m = lr_smem(lsm, s.r);
     const int chunk = blockIdx.x, bh = blockIdx.y, h = bh % s.H, b = bh / s.H;
@@ -307,6 +308,7 @@ __global__ void __launch_bounds__(kBT) lr_bwd_k_kernel(Shape s, const T* __restr
                                                        const float2* __restrict__ tab, float* __restrict__ dk_acc,
                                                        float* __restrict__ dv_acc, float* __restrict__ partPk)
 {
+    chain_begin();
     extern __shared__ float lsm[];
     const LrSmem m = lr_smem(lsm, s.r);
     const int chunk = blockIdx.x, bh = blockIdx.y, h = bh % s.H;
@@ -362,6 +364,7 @@ __global__ void __launch_bounds__(kBT) lr_bwd_k_kernel(Shape s, const T* __restr
 __global__ void reduce_chunks_kernel(Shape s, const float* __restrict__ part, float* __restrict__ out,
                                      bool per_batch)
 {
+    chain_begin();
     const int per = s.r * kDh;
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     const int grp = blockIdx.y;
@@ -431,6 +434,7 @@ __global__ void __launch_bounds__(kBT) sparse_bwd_dq_kernel(Shape s, const T* __
                                                             const float2* __restrict__ tab,
                                                             float* __restrict__ dq_acc)
 {
+    chain_begin();
     extern __shared__ float ssm[];
     const SpSmem m = sp_smem(ssm);
     const int qb = blockIdx.x, bh = blockIdx.y;
@@ -493,6 +497,7 @@ __global__ void __launch_bounds__(kBT) sparse_bwd_dq_kernel(Shape s, const T* __
 __global__ void __launch_bounds__(1024) mask_transpose_kernel(Shape s, const int32_t* __restrict__ kv_idx,
                                                               int32_t* __restrict__ off, int32_t* __restrict__ list)
 {
+    chain_begin();
     extern __shared__ int cur[];
     const int bh = blockIdx.x;
     const int32_t* kv = kv_idx + (size_t)bh * s.nB * s.n_keep;
@@ -536,6 +541,7 @@ __global__ void __launch_bounds__(kBT) sparse_bwd_dkdv_kernel(Shape s, const T* 
                                                               const float2* __restrict__ tab,
                                                               float* __restrict__ dk_acc, float* __restrict__ dv_acc)
 {
+    chain_begin();
     extern __shared__ float ssm[];
     const SpSmem m = sp_smem(ssm);
     const int kb = blockIdx.x, bh = blockIdx.y;
@@ -822,6 +828,7 @@ __global__ void __launch_bounds__(kMT, R <= 32 ? 3 : 1) lr_bwd_q_mma_kernel(Shap
                                                            float* __restrict__ dq_acc, float* __restrict__ dg_h,
                                                            float* __restrict__ partC, float* __restrict__ partPq)
 {
+    chain_begin();
     extern __shared__ __align__(128) uint8_t msm[];
     const uint32_t b0 = smem_u32(msm);
     // layout: X [64] | P [R rows] | C [R rows] | F [64] | dY [64] (rows of 256 B); dU takes F's place
@@ -952,6 +959,7 @@ __global__ void __launch_bounds__(kMT) lr_bwd_k_mma_kernel(Shape s, const __nv_b
                                                            float* __restrict__ dk_acc, float* __restrict__ dv_acc,
                                                            float* __restrict__ partPk)
 {
+    chain_begin();
     extern __shared__ __align__(128) uint8_t msm[];
     const uint32_t b0 = smem_u32(msm);
     // layout: X (k) [64] | V [64] | P [R rows] | dC [R rows]; dU takes V's place: a warp reads only its
@@ -1030,7 +1038,7 @@ cudaError_t launch_lr_mma_r(const Shape& s, const BackwardArgs& a, bool key_side
             e = cudaFuncSetAttribute(lr_bwd_q_mma_kernel<R>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
-        lr_bwd_q_mma_kernel<R><<<chunks, kMT, smem, st>>>(
+        launch_kernel(lr_bwd_q_mma_kernel<R>, chunks, kMT, smem, st,
             s, static_cast<const bf*>(a.q), static_cast<const bf*>(a.P_q), a.C, a.gate, static_cast<const bf*>(a.o_s),
             static_cast<const bf*>(a.dO), a.tab, static_cast<bf*>(a.dOs), a.Dv, a.dq_acc, a.dg_h, a.partC, a.partPq);
     } else {
@@ -1040,7 +1048,7 @@ cudaError_t launch_lr_mma_r(const Shape& s, const BackwardArgs& a, bool key_side
             e = cudaFuncSetAttribute(lr_bwd_k_mma_kernel<R>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
-        lr_bwd_k_mma_kernel<R><<<chunks, kMT, smem, st>>>(s, static_cast<const bf*>(a.k), static_cast<const bf*>(a.v),
+        launch_kernel(lr_bwd_k_mma_kernel<R>, chunks, kMT, smem, st, s, static_cast<const bf*>(a.k), static_cast<const bf*>(a.v),
                                                           static_cast<const bf*>(a.P_k), a.dC, a.tab, a.dk_acc,
                                                           a.dv_acc, a.partPk);
     }
@@ -1071,6 +1079,7 @@ __global__ void __launch_bounds__(kBT) block_order_kernel(Shape s, const T* __re
                                                           T* __restrict__ dOs_b, float* __restrict__ lse_b,
                                                           float* __restrict__ Dv_b)
 {
+    chain_begin();
     const int b = blockIdx.x, bh = blockIdx.y;
     for (int e = threadIdx.x; e < 64 * kDh; e += kBT) {
         const int i = e / kDh, d = e - i * kDh;
@@ -1089,12 +1098,14 @@ __global__ void __launch_bounds__(kBT) block_order_kernel(Shape s, const T* __re
 template <typename T>
 __global__ void store_grad_kernel(size_t n, const float* __restrict__ acc, T* __restrict__ out)
 {
+    chain_begin();
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
         out[e] = from_f<T>(acc[e]);
 }
 
 __global__ void gate_grad_kernel(Shape s, const float* __restrict__ dg_h, float* __restrict__ dgate)
 {
+    chain_begin();
     const int p = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
     if (p >= s.N) return;
     float acc = 0.0f;
@@ -1126,7 +1137,7 @@ cudaError_t launch_backward_t(const Shape& s, const BackwardArgs& a, cudaStream_
     if constexpr (kMma) {
         e = launch_lr_mma(s, a, false, st);
     } else {
-        lr_bwd_q_kernel<T><<<chunks, kBT, lsm, st>>>(s, q, static_cast<const T*>(a.P_q), a.C, a.gate,
+        launch_kernel(lr_bwd_q_kernel<T>, chunks, kBT, lsm, st, s, q, static_cast<const T*>(a.P_q), a.C, a.gate,
                                                      static_cast<const T*>(a.o_s), static_cast<const T*>(a.dO), a.tab,
                                                      static_cast<T*>(a.dOs), a.Dv, a.dq_acc, a.dg_h, a.partC,
                                                      a.partPq);
@@ -1134,19 +1145,19 @@ cudaError_t launch_backward_t(const Shape& s, const BackwardArgs& a, cudaStream_
     }
     if (e != cudaSuccess) return e;
     const dim3 red((s.r * kDh + 255) / 256, s.B * s.H), red_h((s.r * kDh + 255) / 256, s.H);
-    reduce_chunks_kernel<<<red, 256, 0, st>>>(s, a.partC, a.dC, false);
-    reduce_chunks_kernel<<<red_h, 256, 0, st>>>(s, a.partPq, a.dP_q, true);
+    launch_kernel(reduce_chunks_kernel, red, 256, 0, st, s, a.partC, a.dC, false);
+    launch_kernel(reduce_chunks_kernel, red_h, 256, 0, st, s, a.partPq, a.dP_q, true);
     if constexpr (kMma) {
         e = launch_lr_mma(s, a, true, st);
         if (e != cudaSuccess) return e;
     } else {
-        lr_bwd_k_kernel<T><<<chunks, kBT, lsm, st>>>(s, k, v, static_cast<const T*>(a.P_k), a.dC, a.tab, a.dk_acc,
+        launch_kernel(lr_bwd_k_kernel<T>, chunks, kBT, lsm, st, s, k, v, static_cast<const T*>(a.P_k), a.dC, a.tab, a.dk_acc,
                                                      a.dv_acc, a.partPk);
     }
-    reduce_chunks_kernel<<<red_h, 256, 0, st>>>(s, a.partPk, a.dP_k, true);
+    launch_kernel(reduce_chunks_kernel, red_h, 256, 0, st, s, a.partPk, a.dP_k, true);
     // the sparse kernels read v, dO^s, lse and D in block order (copies for cube blocks)
     if (s.cube)
-        block_order_kernel<T><<<blocks, kBT, 0, st>>>(s, static_cast<const T*>(a.dOs), a.lse, a.Dv,
+        launch_kernel(block_order_kernel<T>, blocks, kBT, 0, st, s, static_cast<const T*>(a.dOs), a.lse, a.Dv,
                                                       static_cast<T*>(a.dOs_blk), a.lse_blk, a.Dv_blk);
     const T* vb = static_cast<const T*>(s.cube ? a.v_blk : a.v);
     const T* dOb = static_cast<const T*>(s.cube ? a.dOs_blk : a.dOs);
@@ -1156,7 +1167,7 @@ cudaError_t launch_backward_t(const Shape& s, const BackwardArgs& a, cudaStream_
         e = launch_sparse_bwd_dq_tc(s, qr, kr, vb, dOb, a.kv_idx, lseb, Dvb, a.tab, a.dq_acc, a.dq, a.status, st);
         if (e != cudaSuccess) return e;
     } else {
-        sparse_bwd_dq_kernel<T><<<blocks, kBT, kSpSmemBytes, st>>>(s, qr, kr, vb, a.kv_idx, lseb, Dvb, dOb, a.tab,
+        launch_kernel(sparse_bwd_dq_kernel<T>, blocks, kBT, kSpSmemBytes, st, s, qr, kr, vb, a.kv_idx, lseb, Dvb, dOb, a.tab,
                                                                   a.dq_acc);
     }
     const size_t tsm = sizeof(int) * (size_t)s.nB;
@@ -1164,21 +1175,21 @@ cudaError_t launch_backward_t(const Shape& s, const BackwardArgs& a, cudaStream_
         e = cudaFuncSetAttribute(mask_transpose_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm);
         if (e != cudaSuccess) return e;
     }
-    mask_transpose_kernel<<<s.B * s.H, 1024, tsm, st>>>(s, a.kv_idx, a.tr_off, a.tr_list);
+    launch_kernel(mask_transpose_kernel, s.B * s.H, 1024, tsm, st, s, a.kv_idx, a.tr_off, a.tr_list);
     if constexpr (kMma) {
         e = launch_sparse_bwd_dkdv_tc(s, qr, kr, vb, dOb, a.tr_off, a.tr_list, lseb, Dvb, a.tab, a.dk_acc, a.dv_acc,
                                       a.dk, a.dv, a.status, st);
         if (e != cudaSuccess) return e;
     } else {
-        sparse_bwd_dkdv_kernel<T><<<blocks, kBT, kSpSmemBytes, st>>>(s, qr, kr, vb, a.tr_off, a.tr_list, lseb, Dvb,
+        launch_kernel(sparse_bwd_dkdv_kernel<T>, blocks, kBT, kSpSmemBytes, st, s, qr, kr, vb, a.tr_off, a.tr_list, lseb, Dvb,
                                                                     dOb, a.tab, a.dk_acc, a.dv_acc);
         const size_t nel = (size_t)s.B * s.H * s.N * kDh;
         const int sg = 152 * 8;
-        store_grad_kernel<T><<<sg, 256, 0, st>>>(nel, a.dq_acc, static_cast<T*>(a.dq));
-        store_grad_kernel<T><<<sg, 256, 0, st>>>(nel, a.dk_acc, static_cast<T*>(a.dk));
-        store_grad_kernel<T><<<sg, 256, 0, st>>>(nel, a.dv_acc, static_cast<T*>(a.dv));
+        launch_kernel(store_grad_kernel<T>, sg, 256, 0, st, nel, a.dq_acc, static_cast<T*>(a.dq));
+        launch_kernel(store_grad_kernel<T>, sg, 256, 0, st, nel, a.dk_acc, static_cast<T*>(a.dk));
+        launch_kernel(store_grad_kernel<T>, sg, 256, 0, st, nel, a.dv_acc, static_cast<T*>(a.dv));
     }
-    if (a.dgate) gate_grad_kernel<<<dim3((s.N + 255) / 256, s.B), 256, 0, st>>>(s, a.dg_h, a.dgate);
+    if (a.dgate) launch_kernel(gate_grad_kernel, dim3((s.N + 255) / 256, s.B), 256, 0, st, s, a.dg_h, a.dgate);
     return cudaGetLastError();
 }
 

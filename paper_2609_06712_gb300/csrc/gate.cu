@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(32 * kGateWarps) gate_kernel(long long rows, i
                                                                const T* __restrict__ w, float b,
                                                                float* __restrict__ g)
 {
+    chain_begin();
     const int lane = threadIdx.x & 31;
     const long long stride = (long long)gridDim.x * kGateWarps;
     for (long long row = (long long)blockIdx.x * kGateWarps + (threadIdx.x >> 5); row < rows; row += stride) {
@@ -68,10 +69,10 @@ cudaError_t launch_gate(rola_dtype_t dt, long long rows, int D, const void* X, c
     const long long cap = (long long)nsm * 8;            // 8 CTAs of 8 warps per SM, rows grid-strided
     const int grid = (int)(want < cap ? want : cap);
     if (dt == ROLA_BF16)
-        gate_kernel<__nv_bfloat16><<<grid, 32 * kGateWarps, 0, st>>>(
+        launch_kernel(gate_kernel<__nv_bfloat16>, grid, 32 * kGateWarps, 0, st,
             rows, D, static_cast<const __nv_bfloat16*>(X), static_cast<const __nv_bfloat16*>(w), b, g);
     else
-        gate_kernel<float><<<grid, 32 * kGateWarps, 0, st>>>(rows, D, static_cast<const float*>(X),
+        launch_kernel(gate_kernel<float>, grid, 32 * kGateWarps, 0, st, rows, D, static_cast<const float*>(X),
                                                                static_cast<const float*>(w), b, g);
     return cudaGetLastError();
 }

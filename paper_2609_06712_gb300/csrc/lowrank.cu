@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(256) summary_f32_kernel(Shape s, int tokens_pe
                                                           const float* __restrict__ v, const float* __restrict__ Pk,
                                                           const float2* __restrict__ tab, float* __restrict__ partials)
 {
+    chain_begin();
     extern __shared__ float fsm[];
     const int R = s.r;
     float* Ps = fsm;                           // [R][129]
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(256) summary_f32_kernel(Shape s, int tokens_pe
 __global__ void summary_combine_kernel(Shape s, int nsplit, const float* __restrict__ partials, float* __restrict__ C,
                                        float* __restrict__ z, __nv_bfloat16* __restrict__ Cbf)
 {
+    chain_begin();
     const int bh = blockIdx.y;
     const int per = s.r * kDh + s.r;
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -129,6 +131,7 @@ __global__ void summary_combine_kernel(Shape s, int nsplit, const float* __restr
 // C [B*H][r][128] fp32 -> bf16 [B*H][rp][128], rows r .. rp-1 zero
 __global__ void c_to_bf16_kernel(int r, int rp, int n, const float* __restrict__ C, __nv_bfloat16* __restrict__ Cbf)
 {
+    chain_begin();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;     // index into the padded copy
     if (e >= n) return;
     const int bh = e / (rp * kDh), rest = e - bh * rp * kDh, row = rest / kDh;
@@ -138,7 +141,7 @@ __global__ void c_to_bf16_kernel(int r, int rp, int n, const float* __restrict__
 cudaError_t launch_c_to_bf16(const Shape& s, const float* C, __nv_bfloat16* Cbf, cudaStream_t st)
 {
     int n = s.B * s.H * s.rp * kDh;
-    c_to_bf16_kernel<<<(n + 255) / 256, 256, 0, st>>>(s.r, s.rp, n, C, Cbf);
+    launch_kernel(c_to_bf16_kernel, (n + 255) / 256, 256, 0, st, s.r, s.rp, n, C, Cbf);
     return cudaGetLastError();
 }
 
@@ -153,12 +156,12 @@ cudaError_t launch_lowrank_summary(rola_dtype_t dt, const Shape& s, int nsplit, 
                                    kF32Tile * (s.r + 1));
     cudaError_t e = cudaFuncSetAttribute(summary_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    summary_f32_kernel<<<dim3(nsplit, s.B * s.H), 256, smem, st>>>(s, tps, (const float*)k, (const float*)v,
+    launch_kernel(summary_f32_kernel, dim3(nsplit, s.B * s.H), 256, smem, st, s, tps, (const float*)k, (const float*)v,
                                                                     (const float*)P_k, tab, partials);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     int per = s.r * kDh + s.r;
-    summary_combine_kernel<<<dim3((per + 255) / 256, s.B * s.H), 256, 0, st>>>(s, nsplit, partials, C, z, Cbf);
+    launch_kernel(summary_combine_kernel, dim3((per + 255) / 256, s.B * s.H), 256, 0, st, s, nsplit, partials, C, z, Cbf);
     return cudaGetLastError();
 }
 
@@ -170,6 +173,7 @@ __global__ void __launch_bounds__(256) apply_f32_kernel(Shape s, const float* __
                                                         const float* __restrict__ gate, const float* o_s, float* o,
                                                         const float2* __restrict__ tab)
 {
+    chain_begin();
     extern __shared__ float fsm[];
     const int R = s.r;
     float* Ps = fsm;                        // [R][129]
@@ -236,7 +240,7 @@ cudaError_t launch_lowrank_apply(rola_dtype_t dt, const Shape& s, const void* q,
                                    kBlock * (s.r + 1));
     cudaError_t e = cudaFuncSetAttribute(apply_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    apply_f32_kernel<<<dim3(s.nC, s.B * s.H), 256, smem, st>>>(s, (const float*)q, (const float*)P_q, C, gate,
+    launch_kernel(apply_f32_kernel, dim3(s.nC, s.B * s.H), 256, smem, st, s, (const float*)q, (const float*)P_q, C, gate,
                                                               (const float*)o_s, (float*)o, tab);
     return cudaGetLastError();
 }

@@ -28,6 +28,7 @@ __global__ void __launch_bounds__(256, 2) block_scores_kernel(Shape s, const flo
                                                               const float* __restrict__ kbar,
                                                               float* __restrict__ scores)
 {
+    chain_begin();
     __shared__ __align__(16) float qs[2][kSChunk][kSTile + 4];
     __shared__ __align__(16) float ks[2][kSChunk][kSTile + 4];
     const int bh = blockIdx.z, i0 = blockIdx.y * kSTile, j0 = blockIdx.x * kSTile;
@@ -213,6 +214,7 @@ template <int K>
 __global__ void __launch_bounds__(kTopkWarps * 32) block_topk_kernel(Shape s, const float* __restrict__ scores,
                                                                      int32_t* __restrict__ kv_idx)
 {
+    chain_begin();
     __shared__ uint32_t hist_s[kTopkWarps][256];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t* hist = hist_s[warp];
@@ -345,6 +347,7 @@ __global__ void __launch_bounds__(kTopkWarps * 32) block_topk_kernel(Shape s, co
 __global__ void __launch_bounds__(kTopkWarps * 32) block_topk_long_kernel(Shape s, const float* __restrict__ scores,
                                                                           int32_t* __restrict__ kv_idx)
 {
+    chain_begin();
     extern __shared__ uint32_t tk_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t* hist = tk_smem + warp * 256;
@@ -447,7 +450,7 @@ cudaError_t launch_block_topk(const Shape& s, const float* qbar, const float* kb
                               int32_t* kv_idx, cudaStream_t st)
 {
     const int tj = (s.nB + kSTile - 1) / kSTile, ti = (s.nQ + kSTile - 1) / kSTile;
-    block_scores_kernel<<<dim3(tj, ti, s.B * s.H), 256, 0, st>>>(s, qbar, kbar, scores);
+    launch_kernel(block_scores_kernel, dim3(tj, ti, s.B * s.H), 256, 0, st, s, qbar, kbar, scores);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // registers per lane by the row's length; past 40 a lane too few warps would fit an SM
@@ -458,7 +461,7 @@ cudaError_t launch_block_topk(const Shape& s, const float* qbar, const float* kb
                       : s.nB <= 24 * 32 ? block_topk_kernel<24>
                       : s.nB <= 32 * 32 ? block_topk_kernel<32>
                                         : block_topk_kernel<40>;
-        kernel<<<grid, kTopkWarps * 32, 0, st>>>(s, scores, kv_idx);
+        launch_kernel(kernel, grid, kTopkWarps * 32, 0, st, s, scores, kv_idx);
         return cudaGetLastError();
     }
     const size_t smem = (size_t)kTopkWarps * (256 + s.nB) * 4;
@@ -466,7 +469,7 @@ cudaError_t launch_block_topk(const Shape& s, const float* qbar, const float* kb
         e = cudaFuncSetAttribute(block_topk_long_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    block_topk_long_kernel<<<grid, kTopkWarps * 32, smem, st>>>(s, scores, kv_idx);
+    launch_kernel(block_topk_long_kernel, grid, kTopkWarps * 32, smem, st, s, scores, kv_idx);
     return cudaGetLastError();
 }
 
@@ -477,6 +480,7 @@ cudaError_t launch_block_topk(const Shape& s, const float* qbar, const float* kb
 // the chunk's token count -- the pairwise sum over 128 slots.
 __global__ void qpool128_kernel(Shape s, const float* __restrict__ qsum, float* __restrict__ qbar)
 {
+    chain_begin();
     const int c = blockIdx.x, bh = blockIdx.y, d = threadIdx.x;
     const float* src = qsum + ((size_t)bh * s.nB + 2 * c) * kDh + d;
     const float right = 2 * c + 1 < s.nB ? src[kDh] : 0.0f;
@@ -486,7 +490,7 @@ __global__ void qpool128_kernel(Shape s, const float* __restrict__ qsum, float* 
 
 cudaError_t launch_qpool128(const Shape& s, const float* qsum64, float* qbar128, cudaStream_t st)
 {
-    qpool128_kernel<<<dim3(s.nQ, s.B * s.H), kDh, 0, st>>>(s, qsum64, qbar128);
+    launch_kernel(qpool128_kernel, dim3(s.nQ, s.B * s.H), kDh, 0, st, s, qsum64, qbar128);
     return cudaGetLastError();
 }
 

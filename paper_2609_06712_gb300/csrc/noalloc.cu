@@ -62,6 +62,7 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 // partials, so they become NaN.  Nothing is written when the status word is clear.
 __global__ void poison_on_timeout_kernel(const DeviceStatus* status, float* C, int nC, float* z, int nz)
 {
+    chain_begin();
     if (status->code == 0) return;
     const float nan = __int_as_float(0x7fc00000);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nC + nz; i += gridDim.x * blockDim.x) {
@@ -99,8 +100,7 @@ extern "C" rola_status_t rola_lowrank_summary_static(const rola_config_t* cfg, c
     float2* tab = reinterpret_cast<float2*>(b + head);
     float* partials = reinterpret_cast<float*>(b + head + table);
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(status, 0, sizeof(DeviceStatus), cs) != cudaSuccess) return ROLA_ERR_CUDA;
-    if (launch_rope_table(*cfg, tab, cs) != cudaSuccess) return ROLA_ERR_CUDA;
+    if (launch_rope_table(*cfg, tab, status, cs) != cudaSuccess) return ROLA_ERR_CUDA;
     if (cfg->dtype == ROLA_BF16) {
         const size_t cap = fit - bh + 1;                                    // CTAs whose slots fit
         const int ctas = prepass_ctas(s, cap < (size_t)kMaxPrepassCtas ? (int)cap : kMaxPrepassCtas);
@@ -110,7 +110,7 @@ extern "C" rola_status_t rola_lowrank_summary_static(const rola_config_t* cfg, c
             launch_prepass_combine(s, ctas, partials, C, z, nullptr, cs) != cudaSuccess)
             return ROLA_ERR_CUDA;
         const int nC = (int)(bh * (size_t)s.r * kDh), nz = z ? (int)(bh * (size_t)s.r) : 0;
-        poison_on_timeout_kernel<<<(nC + nz + 255) / 256 < 1024 ? (nC + nz + 255) / 256 : 1024, 256, 0, cs>>>(
+        launch_kernel(poison_on_timeout_kernel, (nC + nz + 255) / 256 < 1024 ? (nC + nz + 255) / 256 : 1024, 256, 0, cs,
             status, C, nC, z, nz);
         if (cudaGetLastError() != cudaSuccess) return ROLA_ERR_CUDA;
     } else {

@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(kThreads, 1) out_proj_kernel(const __grid_cons
     __syncthreads();
     fence_after_sync();
     const uint32_t tmem = cb.tmem_base;
+    chain_begin();
     volatile int* abort = &cb.abort;
     const uint64_t limit = p.wait_limit_ns;
 
@@ -310,6 +311,7 @@ __global__ void __launch_bounds__(256) out_proj_f32_kernel(int N, int H, int d_m
                                                            const float* __restrict__ W, const float* __restrict__ bias,
                                                            float* __restrict__ Y)
 {
+    chain_begin();
     __shared__ float as[kF32Chunk][kF32Tile + 1];
     __shared__ float bs[kF32Chunk][kF32Tile + 1];
     const int b = blockIdx.z, n0 = blockIdx.y * kF32Tile, f0 = blockIdx.x * kF32Tile;
@@ -351,7 +353,7 @@ cudaError_t launch_out_proj_f32(int B, int N, int H, int d_model, const float* O
                                 float* Y, cudaStream_t st)
 {
     dim3 grid((d_model + kF32Tile - 1) / kF32Tile, (N + kF32Tile - 1) / kF32Tile, B);
-    out_proj_f32_kernel<<<grid, 256, 0, st>>>(N, H, d_model, O, W, bias, Y);
+    launch_kernel(out_proj_f32_kernel, grid, 256, 0, st, N, H, d_model, O, W, bias, Y);
     return cudaGetLastError();
 }
 
@@ -398,7 +400,7 @@ cudaError_t launch_out_proj(int B, int N, int H, int d_model, const void* O, con
     e = cudaFuncSetAttribute(out_proj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int grid = p.tiles < nsm ? p.tiles : nsm;
-    out_proj_kernel<<<grid, kThreads, smem, st>>>(mo, mw, my, p);
+    launch_kernel(out_proj_kernel, grid, kThreads, smem, st, mo, mw, my, p);
     return cudaGetLastError();
 }
 

@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<R>::kCtasPerSm) prepass_kernel(
         if (fuse) tma_prefetch_desc(&map_q);
     }
     __syncthreads();
+    chain_begin();
 
     // loads of the j-th half-stage of the range into stage j % S: lane 0 of
     // warps 0, 1, 2 issue the k, v, q boxes; thread 0 also arms the barrier
@@ -472,6 +473,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<R>::kCtasPerSm) prepass_kernel(
 __global__ void prepass_combine_kernel(Shape s, int ctas, int units, const float* __restrict__ partials,
                                        float* __restrict__ C, float* __restrict__ z, __nv_bfloat16* __restrict__ Cbf)
 {
+    chain_begin();
     const int bh = blockIdx.y;
     const int per = s.rp * kDh + s.rp;                 // one partial slot (rp rows)
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -498,7 +500,7 @@ cudaError_t launch_ra(const CUtensorMap& mq, const CUtensorMap& mk, const CUtens
     cudaError_t e = cudaFuncSetAttribute(prepass_kernel<R, Act>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)lay.total);
     if (e != cudaSuccess) return e;
-    prepass_kernel<R, Act><<<ctas, kThreads, lay.total, st>>>(mq, mk, mv, p);
+    launch_kernel(prepass_kernel<R, Act>, ctas, kThreads, lay.total, st, mq, mk, mv, p);
     return cudaGetLastError();
 }
 
@@ -568,7 +570,7 @@ cudaError_t launch_prepass_combine(const Shape& s, int ctas, const float* partia
 {
     const int per = s.rp * kDh + s.rp;
     const int units = s.B * s.H * s.nC;
-    prepass_combine_kernel<<<dim3((per + 255) / 256, s.B * s.H), 256, 0, st>>>(s, ctas, units, partials, C, z, Cbf);
+    launch_kernel(prepass_combine_kernel, dim3((per + 255) / 256, s.B * s.H), 256, 0, st, s, ctas, units, partials, C, z, Cbf);
     return cudaGetLastError();
 }
 

@@ -100,6 +100,7 @@ __global__ void __launch_bounds__(32 * Layout<R>::warps, 1) readout_kernel(const
         tma_prefetch_desc(&map_os);
         tma_prefetch_desc(&map_o);
     }
+    chain_begin();
     bool ok = true;
     int i = 0;                                       // tiles of this warp so far (buffer and phase)
     int q_issued = 0, o_issued = 0;                  // loads of this warp so far
@@ -273,7 +274,7 @@ cudaError_t launch_ra(const CUtensorMap& mq, const CUtensorMap& mos, const CUten
     cudaError_t e =
         cudaFuncSetAttribute(readout_kernel<R, Act>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::total);
     if (e != cudaSuccess) return e;
-    readout_kernel<R, Act><<<ctas, 32 * L::warps, L::total, st>>>(mq, mos, mo, p);
+    launch_kernel(readout_kernel<R, Act>, ctas, 32 * L::warps, L::total, st, mq, mos, mo, p);
     return cudaGetLastError();
 }
 

@@ -4,40 +4,51 @@
 // (2m, 2m+1); the first d_t/2 pairs turn with the temporal position, the next
 // d_x/2 with the row, the rest with the column; within an axis the i-th pair
 // turns by pos * theta^(-2i/d_axis).  The table holds (cos, sin) in fp32,
-// evaluated in fp64 once per call.
+// evaluated in fp64 once per call (frequencies on the host, angles and (cos, sin) on the GPU).
+#include <math.h>
+
 #include "common.cuh"
 
 namespace rola {
 
-__global__ void rope_table_kernel(float2* __restrict__ tab, int T, int Hh, int Ww, int d_t, int d_x, int d_y,
-                                  int off_t, int off_x, int off_y, double theta)
+// theta^(-2i/d_axis) of every pair, in fp64.  Computed on the host: 64 of them
+// serve a whole call, and a pow per table entry on the GPU's few fp64 lanes was most of
+// the 11 us that the table used to take.
+struct Frequencies {
+    double f[kPairs];
+};
+
+// One CTA per table row; the row's axis owns pairs m0 .. m0 + count - 1, the others keep (1, 0).
+__global__ void rope_table_kernel(float2* __restrict__ tab, int T, int Hh, int pt, int px, int off_t, int off_x,
+                                  int off_y, const __grid_constant__ Frequencies freq, DeviceStatus* status)
 {
-    int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    int rows = T + Hh + Ww;
-    if (idx >= rows * kPairs) return;
-    int row = idx / kPairs, m = idx % kPairs;
-    int pt = d_t / 2, px = d_x / 2;
-    int axis = m < pt ? 0 : (m < pt + px ? 1 : 2);
-    int row_axis = row < T ? 0 : (row < T + Hh ? 1 : 2);
+    chain_begin();
+    const int row = blockIdx.x, m = threadIdx.x;
+    if (row == 0) reinterpret_cast<int*>(status)[m] = 0;
+    static_assert(sizeof(DeviceStatus) == kPairs * sizeof(int), "one status word a thread");
+    const int axis = row < T ? 0 : (row < T + Hh ? 1 : 2);
+    const int m0 = axis == 0 ? 0 : (axis == 1 ? pt : pt + px);
+    const int count = axis == 0 ? pt : (axis == 1 ? px : kPairs - pt - px);
+    const int pos = axis == 0 ? row + off_t : (axis == 1 ? row - T + off_x : row - T - Hh + off_y);
+    // thread i takes pair m0 + i (mod 64), so that the fp64 work of a row fills as few warps as it can
+    const int pair = (m0 + m) & (kPairs - 1);
     float2 out = make_float2(1.0f, 0.0f);
-    if (axis == row_axis) {
-        int i = axis == 0 ? m : (axis == 1 ? m - pt : m - pt - px);
-        int d_axis = axis == 0 ? d_t : (axis == 1 ? d_x : d_y);
-        int pos = axis == 0 ? row + off_t : (axis == 1 ? row - T + off_x : row - T - Hh + off_y);
-        double freq = pow(theta, -2.0 * (double)i / (double)d_axis);
+    if (m < count) {
         double s, c;
-        sincos((double)pos * freq, &s, &c);
+        sincos((double)pos * freq.f[pair], &s, &c);
         out = make_float2((float)c, (float)s);
     }
-    tab[idx] = out;
+    tab[row * kPairs + pair] = out;
 }
 
-cudaError_t launch_rope_table(const rola_config_t& cfg, float2* tab, cudaStream_t st)
+cudaError_t launch_rope_table(const rola_config_t& cfg, float2* tab, DeviceStatus* status, cudaStream_t st)
 {
-    int n = (cfg.T + cfg.Hh + cfg.Ww) * kPairs;
-    rope_table_kernel<<<(n + 255) / 256, 256, 0, st>>>(tab, cfg.T, cfg.Hh, cfg.Ww, cfg.rope_split[0],
-                                                       cfg.rope_split[1], cfg.rope_split[2], cfg.pos_offset[0],
-                                                       cfg.pos_offset[1], cfg.pos_offset[2], cfg.rope_theta);
+    Frequencies freq;
+    for (int axis = 0, m = 0; axis < 3; ++axis)
+        for (int i = 0; i < cfg.rope_split[axis] / 2; ++i, ++m)
+            freq.f[m] = pow(cfg.rope_theta, -2.0 * (double)i / (double)cfg.rope_split[axis]);
+    launch_kernel(rope_table_kernel, cfg.T + cfg.Hh + cfg.Ww, kPairs, 0, st, tab, cfg.T, cfg.Hh, cfg.rope_split[0] / 2,
+                  cfg.rope_split[1] / 2, cfg.pos_offset[0], cfg.pos_offset[1], cfg.pos_offset[2], freq, status);
     return cudaGetLastError();
 }
 
@@ -91,6 +102,7 @@ __global__ void __launch_bounds__(256) rope_pool_kernel(Shape s, const T* __rest
                                                         T* __restrict__ qr, T* __restrict__ kr, T* __restrict__ vp,
                                                         float* __restrict__ qbar, float* __restrict__ kbar)
 {
+    chain_begin();
     using Raw = typename Vec4<T>::Raw;
     __shared__ __align__(16) float nodes[8][kDh];            // level-3 nodes of the pairwise sum, slot order
     const int blk = blockIdx.x, bh = blockIdx.y, z = blockIdx.z;
@@ -202,7 +214,7 @@ cudaError_t launch_rope_pool_t(const Shape& s, const void* q, const void* k, con
 {
     const dim3 grid(s.nB, s.B * s.H, s.cube && v ? 3 : 2);
     auto kernel = s.cube ? rope_pool_kernel<T, true> : rope_pool_kernel<T, false>;
-    kernel<<<grid, 256, 0, st>>>(s, (const T*)q, (const T*)k, (const T*)v, tab, (T*)qr, (T*)kr, (T*)vp, qbar, kbar);
+    launch_kernel(kernel, grid, 256, 0, st, s, (const T*)q, (const T*)k, (const T*)v, tab, (T*)qr, (T*)kr, (T*)vp, qbar, kbar);
     return cudaGetLastError();
 }
 

@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(kF32Threads, 1) sparse_attn_f32_kernel(Shape s
                                                                          const int32_t* __restrict__ kv_idx,
                                                                          float* __restrict__ o, float* __restrict__ lse)
 {
+    chain_begin();
     extern __shared__ __align__(16) uint8_t fsm[];
     F32Smem& sm = *reinterpret_cast<F32Smem*>(fsm);
     const int qb = blockIdx.x, bh = blockIdx.y, tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
@@ -196,7 +197,7 @@ cudaError_t launch_sparse_attn(rola_dtype_t dt, const Shape& s, const void* qr, 
     auto kernel = s.cube ? sparse_attn_f32_kernel<true> : sparse_attn_f32_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(F32Smem));
     if (e != cudaSuccess) return e;
-    kernel<<<dim3(s.nB, s.B * s.H), kF32Threads, sizeof(F32Smem), st>>>(s, (const float*)qr, (const float*)kr,
+    launch_kernel(kernel, dim3(s.nB, s.B * s.H), kF32Threads, sizeof(F32Smem), st, s, (const float*)qr, (const float*)kr,
                                                                        (const float*)v, kv_idx, (float*)o_s, lse);
     return cudaGetLastError();
 }

@@ -247,6 +247,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
     __syncthreads();
     fence_after_sync();
     const uint32_t tmem = sm.tmem_base;
+    chain_begin();
     volatile int* abort = &sm.abort;
 
     if constexpr (QN == 128) {
@@ -619,7 +620,7 @@ cudaError_t launch_rows(const Shape& s, const void* qr, const void* kr, const vo
     auto kernel = sparse_attn_rows_kernel<QN, kCube>;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kernel<<<grid, kThreads, smem, st>>>(mq, mk, mv, p);
+    launch_kernel(kernel, grid, kThreads, smem, st, mq, mk, mv, p);
     return cudaGetLastError();
 }
 

@@ -247,6 +247,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
     __syncthreads();
     fence_after_sync();
     const uint32_t tmem = sm.tmem_base;
+    chain_begin();
     volatile int* abort = &sm.abort;
 
     if (warp == kProdAWarp || warp == kProdBWarp) {
@@ -500,6 +501,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
     __syncthreads();
     fence_after_sync();
     const uint32_t tmem = sm.tmem_base;
+    chain_begin();
     volatile int* abort = &sm.abort;
 
     if (warp == kProdAWarp || warp == kProdBWarp) {
@@ -744,7 +746,7 @@ cudaError_t launch(Kernel kernel, size_t smem, const CUtensorMap (&m)[4], const 
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kernel<<<p.total_items < nsm ? p.total_items : nsm, kThreads, smem, st>>>(m[0], m[1], m[2], m[3], p);
+    launch_kernel(kernel, p.total_items < nsm ? p.total_items : nsm, kThreads, smem, st, m[0], m[1], m[2], m[3], p);
     return cudaGetLastError();
 }
 
