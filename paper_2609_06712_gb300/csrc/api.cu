@@ -299,6 +299,7 @@ rola_status_t forward_impl(const rola_config_t* cfg, const void* q, const void* 
     Workspace w = layout(*cfg);
     Shape s = make_shape(*cfg);
     int32_t* kv = kv_idx_out ? kv_idx_out : at<int32_t>(ws, w.kv_idx);
+    float* C = C_out ? C_out : at<float>(ws, w.C);
     ROLA_TRY(mark(0));
     ROLA_CHECK(prologue(*cfg, ws, w, st));
     if (cfg->dtype == ROLA_BF16 && s.cube) {
@@ -312,7 +313,7 @@ rola_status_t forward_impl(const rola_config_t* cfg, const void* q, const void* 
                                 nullptr, at<float>(ws, w.partials), at<DeviceStatus>(ws, w.status), st));
         ROLA_TRY(mark(1));
         ROLA_TRY(select_blocks(s, w, kv, ws, st));
-        ROLA_TRY(launch_prepass_combine(s, ctas, at<float>(ws, w.partials), at<float>(ws, w.C), at<float>(ws, w.z),
+        ROLA_TRY(launch_prepass_combine(s, ctas, at<float>(ws, w.partials), C, at<float>(ws, w.z),
                                         at<__nv_bfloat16>(ws, w.Cbf), st));
     } else if (cfg->dtype == ROLA_BF16) {
         // stage 1: one pass over q, k, v -> q^r, k^r, block means, summary partials;
@@ -324,24 +325,21 @@ rola_status_t forward_impl(const rola_config_t* cfg, const void* q, const void* 
                                 at<float>(ws, w.partials), at<DeviceStatus>(ws, w.status), st));
         ROLA_TRY(mark(1));
         ROLA_TRY(select_blocks(s, w, kv, ws, st));
-        ROLA_TRY(launch_prepass_combine(s, ctas, at<float>(ws, w.partials), at<float>(ws, w.C), at<float>(ws, w.z),
+        ROLA_TRY(launch_prepass_combine(s, ctas, at<float>(ws, w.partials), C, at<float>(ws, w.z),
                                         at<__nv_bfloat16>(ws, w.Cbf), st));
     } else {
         // stage 1: the block mask; stage 2: the summary
         ROLA_CHECK(run_mask(*cfg, s, w, q, k, v, true, kv, ws, st));
         ROLA_TRY(mark(1));
-        ROLA_CHECK(run_summary(*cfg, s, w, k, v, P_k, at<float>(ws, w.C), at<float>(ws, w.z),
+        ROLA_CHECK(run_summary(*cfg, s, w, k, v, P_k, C, at<float>(ws, w.z),
                                at<__nv_bfloat16>(ws, w.Cbf), ws, st));
     }
-    if (C_out)
-        ROLA_TRY(cudaMemcpyAsync(C_out, at<float>(ws, w.C), sizeof(float) * (size_t)s.B * s.H * s.r * kDh,
-                                 cudaMemcpyDeviceToDevice, st));
     void* os = o_s_out ? o_s_out : o;
     ROLA_TRY(mark(2));
     ROLA_TRY(launch_sparse_attn(cfg->dtype, s, at<void>(ws, w.qr), at<void>(ws, w.kr), sparse_v(s, w, v, ws), kv, os,
                                 lse_out, at<DeviceStatus>(ws, w.status), st));
     ROLA_TRY(mark(3));
-    ROLA_TRY(launch_lowrank_apply(cfg->dtype, s, q, P_q, at<float>(ws, w.C), at<__nv_bfloat16>(ws, w.Cbf), gate, os,
+    ROLA_TRY(launch_lowrank_apply(cfg->dtype, s, q, P_q, C, at<__nv_bfloat16>(ws, w.Cbf), gate, os,
                                   o, at<float2>(ws, w.table), at<DeviceStatus>(ws, w.status), st));
     ROLA_TRY(mark(4));
     return ROLA_OK;

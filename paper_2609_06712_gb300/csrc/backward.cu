@@ -361,10 +361,13 @@ __global__ void __launch_bounds__(kBT) lr_bwd_k_kernel(Shape s, const T* __restr
 
 // out[g][e] = sum over the groups' slots in order: slot (b, h, i), i < slots, for
 // out[h] (per_batch = true: P_q, P_k summed over the batch) or for out[bh].
-__global__ void reduce_chunks_kernel(Shape s, int slots, const float* __restrict__ part, float* __restrict__ out,
-                                     bool per_batch)
+// (blockIdx.z picks the first or the second of two such reductions)
+__global__ void reduce_chunks_kernel(Shape s, int slots, const float* __restrict__ part0, float* __restrict__ out0,
+                                     const float* __restrict__ part1, float* __restrict__ out1, bool per_batch)
 {
     chain_begin();
+    const float* part = blockIdx.z ? part1 : part0;
+    float* out = blockIdx.z ? out1 : out0;
     const int per = s.r * kDh;
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     const int grp = blockIdx.y;
@@ -1237,9 +1240,8 @@ cudaError_t launch_backward_t(const Shape& s, const BackwardArgs& a, cudaStream_
     }
     if (e != cudaSuccess) return e;
     const int slots = kMma ? (s.nC + lr_group(s) - 1) / lr_group(s) : s.nC;   // partials of a head
-    const dim3 red((s.r * kDh + 255) / 256, s.B * s.H), red_h((s.r * kDh + 255) / 256, s.H);
-    launch_kernel(reduce_chunks_kernel, red, 256, 0, st, s, slots, a.partC, a.dC, false);
-    launch_kernel(reduce_chunks_kernel, red_h, 256, 0, st, s, slots, a.partPq, a.dP_q, true);
+    const dim3 red((s.r * kDh + 255) / 256, s.B * s.H), red_h((s.r * kDh + 255) / 256, s.H, 2);
+    launch_kernel(reduce_chunks_kernel, red, 256, 0, st, s, slots, a.partC, a.dC, nullptr, nullptr, false);
     if constexpr (kMma) {
         e = launch_lr_mma(s, a, true, st);
         if (e != cudaSuccess) return e;
@@ -1247,7 +1249,7 @@ cudaError_t launch_backward_t(const Shape& s, const BackwardArgs& a, cudaStream_
         launch_kernel(lr_bwd_k_kernel<T>, chunks, kBT, lsm, st, s, k, v, static_cast<const T*>(a.P_k), a.dC, a.tab, a.dk_acc,
                                                      a.dv_acc, a.partPk);
     }
-    launch_kernel(reduce_chunks_kernel, red_h, 256, 0, st, s, slots, a.partPk, a.dP_k, true);
+    launch_kernel(reduce_chunks_kernel, red_h, 256, 0, st, s, slots, a.partPq, a.dP_q, a.partPk, a.dP_k, true);
     // the sparse kernels read v, dO^s, lse and D in block order (copies for cube blocks)
     if (s.cube)
         launch_kernel(block_order_kernel<T>, blocks, kBT, 0, st, s, static_cast<const T*>(a.dOs), a.lse, a.Dv,

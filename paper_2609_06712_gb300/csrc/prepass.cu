@@ -16,8 +16,9 @@
 //
 // A unit is processed as two 32-token halves, each a stage of the TMA ring
 // (k, v and q boxes of 32 x 128, 8 KB each), which keeps a CTA small enough
-// that two fit on an SM for r <= 48 (16 warps per SM hide the latency of the
-// dependent MMA and rotation chains).  Per half, 8 warps:
+// that two fit on an SM for r <= 64 (16 warps per SM hide the latency of the
+// dependent MMA and rotation chains; r = 64 with one CTA an SM took 914 us for the
+// summary of 40 heads and 75600 tokens, 562 with two).  Per half, 8 warps:
 //   rotate q, k (warp w = token rows 4w .. 4w + 3, lane = 4 coordinates),
 //   store q^r, k^r, pool; U = K P_k^T (mma.sync; warp = 16 tokens x a quarter
 //   or half of the r columns); k~ = R_r SiLU(U) to shared memory; the half's
@@ -66,7 +67,7 @@ struct Cfg {
     static constexpr int NSPLIT = NT % 4 == 0 ? 4 : 2;           // column groups of U
     static constexpr int NTW = NT / NSPLIT;                      // n-tiles per warp
     static constexpr int KT = 2 * R + 16;                        // bytes per k~ row (padded)
-    static constexpr int kCtasPerSm = R <= 48 ? 2 : 1;
+    static constexpr int kCtasPerSm = R <= 64 ? 2 : 1;
 };
 
 struct Layout {
@@ -74,8 +75,8 @@ struct Layout {
     uint32_t stage_bytes, P, kt, part, zsm, bars, total;
     __host__ __device__ Layout(int R, bool fuse)
     {
-        const bool two = R <= 48;                                 // two CTAs per SM
-        stages = two ? (fuse ? 3 : 4) : (fuse ? 6 : 8);
+        const bool two = R <= 64;                                 // two CTAs per SM
+        stages = two ? (fuse ? (R <= 48 ? 3 : 2) : 4) : (fuse ? 6 : 8);
         stage_bytes = fuse ? 3 * kHalf : 2 * kHalf;
         P = stages * stage_bytes;                                 // P_k of the current head, r rows x 256 B
         kt = P + R * 256;                                         // k~, two buffers of 32 rows
@@ -521,7 +522,7 @@ int prepass_ctas(const Shape& s, int max_ctas)
                                                    cudaSuccess)
         return 0;
     const long long units = (long long)s.B * s.H * s.nC;
-    long long g = (long long)nsm * (s.rp <= 48 ? 2 : 1);     // CTAs per SM as Cfg<R>::kCtasPerSm
+    long long g = (long long)nsm * (s.rp <= 64 ? 2 : 1);     // CTAs per SM as Cfg<R>::kCtasPerSm
     if (g > max_ctas) g = max_ctas;
     if (g > kMaxPrepassCtas) g = kMaxPrepassCtas;
     if (g > units) g = units;

@@ -59,6 +59,7 @@ struct Params {
     const float2* tab;
     DeviceStatus* status;
     int tiles;                // 16-token tiles of a head
+    int splits;               // > 0: CTAs per head, none of which meets two heads
 };
 
 // SiLU with the MUFU exponential; the kernel is instantiated for it and for
@@ -89,7 +90,12 @@ __global__ void __launch_bounds__(32 * Layout<R>::warps, 1) readout_kernel(const
     const uint32_t q_full = sbase + L::bars + warp * (1 + OB) * 8, o_full = q_full + 8;
     volatile int* abort = reinterpret_cast<volatile int*>(smem + L::abort);
     const long long total = (long long)s.B * s.H * p.tiles;
-    const long long u0 = (long long)blockIdx.x * total / gridDim.x, u1 = (long long)(blockIdx.x + 1) * total / gridDim.x;
+    long long u0 = (long long)blockIdx.x * total / gridDim.x, u1 = (long long)(blockIdx.x + 1) * total / gridDim.x;
+    if (p.splits > 0) {
+        const int bh = blockIdx.x / p.splits, i = blockIdx.x - bh * p.splits;
+        u0 = (long long)bh * p.tiles + (long long)i * p.tiles / p.splits;
+        u1 = (long long)bh * p.tiles + (long long)(i + 1) * p.tiles / p.splits;
+    }
     const int hw = s.Hh * s.Ww;
 
     if (tid == 0) {
@@ -299,7 +305,12 @@ cudaError_t launch_readout(const Shape& s, const void* q, const void* P_q, const
     e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const long long total = (long long)s.B * s.H * tiles;
-    const int ctas = total < nsm ? (int)total : nsm;
+    // Small layers: a CTA that meets two heads loads two sets of weights one after the other, so where
+    // whole CTAs per head leave every warp at most one tile, they are dealt out that way.
+    const int heads = s.B * s.H, warps = s.rp <= 64 ? 16 : 12;                  // Layout<R>::warps
+    const int splits = heads <= nsm ? (nsm / heads < tiles ? nsm / heads : tiles) : 0;
+    const bool whole = splits > 0 && (tiles + splits - 1) / splits <= warps;
+    const int ctas = whole ? heads * splits : (total < nsm ? (int)total : nsm);
     CUtensorMap mq, mos, mo;
     if (!make_block_map(&mq, q, s, kTile) || !make_block_map(&mos, o_s, s, kTile) || !make_block_map(&mo, o, s, kTile))
         return cudaErrorInvalidValue;
@@ -311,6 +322,7 @@ cudaError_t launch_readout(const Shape& s, const void* q, const void* P_q, const
     p.tab = tab;
     p.status = status;
     p.tiles = tiles;
+    p.splits = whole ? splits : 0;
     switch (s.rp) {
         case 16: return launch_r<16>(mq, mos, mo, p, ctas, st);
         case 32: return launch_r<32>(mq, mos, mo, p, ctas, st);
