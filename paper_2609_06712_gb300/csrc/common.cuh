@@ -313,6 +313,14 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t& a, uint32_t& 
                  : "=r"(a), "=r"(b), "=r"(c), "=r"(d) : "r"(addr));
 }
 
+// The four 8 x 8 blocks of ldsm_x4's layout, from registers to shared memory.
+__device__ __forceinline__ void stsm_x4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};\n" ::"r"(addr), "r"(a), "r"(b), "r"(c),
+                 "r"(d)
+                 : "memory");
+}
+
 // D += A(16x16 bf16, row) * B(16x8 bf16, col), fp32 accumulate.
 __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                          uint32_t b0, uint32_t b1)
@@ -341,7 +349,8 @@ __device__ __forceinline__ float fast_exp2(float x)
     return y;
 }
 
-__device__ __forceinline__ float silu(float x) { return x / (1.0f + __expf(-x)); }
+// SiLU of a feature that enters a product in bf16: the approximate divide.
+__device__ __forceinline__ float silu(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
 
 // The feature maps of the activation ablation other than SiLU (Tab. abl_activation),
 // chosen at run time by `kind` (a rola_lowrank_act_t).  tanhf and erff are CUDA's
@@ -358,6 +367,23 @@ struct ActAblation {
         }
     }
 };
+
+// How a bf16 kernel evaluates a pair of features.  The kernels are instantiated for the
+// default, SiLU with the rotation outside, and for any other map or placement.
+struct SiluOutside {
+    __device__ SiluOutside(const Shape&) {}
+    __device__ float2 operator()(float u0, float u1, float2 cs) const { return rope_rotate(silu(u0), silu(u1), cs); }
+};
+struct AnyFeature {
+    int mode, kind;
+    __device__ AnyFeature(const Shape& s) : mode(s.lr_rope), kind(s.lr_act) {}
+    __device__ float operator()(float x) const { return kind == ROLA_LOWRANK_ACT_SILU ? silu(x) : ActAblation{kind}(x); }
+    __device__ float2 operator()(float u0, float u1, float2 cs) const { return lowrank_pair(u0, u1, cs, mode, *this); }
+};
+inline bool default_feature(const Shape& s)
+{
+    return s.lr_act == ROLA_LOWRANK_ACT_SILU && s.lr_rope == ROLA_LOWRANK_ROPE_OUTSIDE;
+}
 
 // Byte offset of 16-byte chunk c of row r in a [rows][128 bf16] tile with the
 // chunk index XOR-swizzled by the row (conflict-free ldmatrix on 8-row groups).

@@ -132,14 +132,7 @@ __device__ __forceinline__ uint2 lds64(uint32_t a)
 }
 
 
-// SiLU with the approximate divide (the features enter the MMA in bf16).  The
-// kernel is instantiated for it and for ActAblation (the other feature maps).
-struct SiluFast {
-    int kind;    // always ROLA_LOWRANK_ACT_SILU
-    __device__ float operator()(float x) const { return __fdividef(x, 1.0f + __expf(-x)); }
-};
-
-template <int R, typename Act>
+template <int R, typename Feature>
 __global__ void __launch_bounds__(kThreads, Cfg<R>::kCtasPerSm) prepass_kernel(
     const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
     const __grid_constant__ CUtensorMap map_v, const Params p)
@@ -160,7 +153,8 @@ __global__ void __launch_bounds__(kThreads, Cfg<R>::kCtasPerSm) prepass_kernel(
     float* zsm = reinterpret_cast<float*>(smem + lay.zsm);
     const uint32_t full0 = sbase + lay.bars;
     volatile int* abort = reinterpret_cast<volatile int*>(smem + lay.bars + kMaxStages * 8);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // (warp: warp-uniform)
+    const Feature feature(s);
     const int u0 = (int)((long long)blockIdx.x * p.units / gridDim.x);
     const int u1 = (int)((long long)(blockIdx.x + 1) * p.units / gridDim.x);
     const int count = 2 * (u1 - u0);                // half-stages of this CTA
@@ -328,15 +322,31 @@ __global__ void __launch_bounds__(kThreads, Cfg<R>::kCtasPerSm) prepass_kernel(
                 advance(8, t, x, y);
             }
         }
-        // (cos, sin) of the rotation's pairs for this thread's four rows
+        // (cos, sin) of the rotation's pairs for this warp's four rows; along a grid row only the
+        // column's pairs change
         float2 cs[4][2];
         if (fuse) {
             int t = rt_t, x = rt_x, y = rt_y;
+            const float2* r0 = p.tab + table_row(axis[0], t, x, y) * kPairs + cq * 2;
+            const float2* r1 = p.tab + table_row(axis[1], t, x, y) * kPairs + cq * 2 + 1;
+            cs[0][0] = __ldg(r0);
+            cs[0][1] = __ldg(r1);
+            if (y + 3 < s.Ww) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+                for (int j = 1; j < 4; ++j) {
+                    cs[j][0] = cs[0][0];
+                    cs[j][1] = cs[0][1];
+                    if (axis[0] == 2) cs[j][0] = __ldg(r0 + j * kPairs);
+                    if (axis[1] == 2) cs[j][1] = __ldg(r1 + j * kPairs);
+                }
+            } else {
 #pragma unroll
-                for (int q = 0; q < 2; ++q) cs[j][q] = __ldg(p.tab + table_row(axis[q], t, x, y) * kPairs + cq * 2 + q);
-                advance(1, t, x, y);
+                for (int j = 1; j < 4; ++j) {
+                    advance(1, t, x, y);
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+                        cs[j][q] = __ldg(p.tab + table_row(axis[q], t, x, y) * kPairs + cq * 2 + q);
+                }
             }
         }
         advance(kHalfRows, kt_t, kt_x, kt_y);          // the next half's positions
@@ -354,13 +364,20 @@ __global__ void __launch_bounds__(kThreads, Cfg<R>::kCtasPerSm) prepass_kernel(
                     wk[j] = lds64(kb + a);
                 }
                 float yq[4][4], yk[4][4];
+                const size_t go = ((size_t)bh * s.N + n_half + 4 * warp) * kDh + cq * 4;
+                if (n_half + kHalfRows <= s.N) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int n = n_half + 4 * warp + j;
-                    const bool valid = n < s.N;
-                    const size_t go = ((size_t)bh * s.N + (valid ? n : 0)) * kDh + cq * 4;
-                    rotate4(wq[j], cs[j], p.qr + go, valid, yq[j]);
-                    rotate4(wk[j], cs[j], p.kr + go, valid, yk[j]);
+                    for (int j = 0; j < 4; ++j) {
+                        rotate4(wq[j], cs[j], p.qr + go + j * kDh, true, yq[j]);
+                        rotate4(wk[j], cs[j], p.kr + go + j * kDh, true, yk[j]);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const bool valid = n_half + 4 * warp + j < s.N;
+                        rotate4(wq[j], cs[j], p.qr + go + j * kDh, valid, yq[j]);
+                        rotate4(wk[j], cs[j], p.kr + go + j * kDh, valid, yk[j]);
+                    }
                 }
                 float4 nq, nk;                           // (y0 + y1) + (y2 + y3) per coordinate
                 nq.x = (yq[0][0] + yq[1][0]) + (yq[2][0] + yq[3][0]);
@@ -408,7 +425,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<R>::kCtasPerSm) prepass_kernel(
                     for (int j = 0; j < NTW; ++j) {
                         const int nt = cg * NTW + j;
                         const float2 cs2 = valid ? kcs[hr][j] : make_float2(0.0f, 0.0f);
-                        const float2 y = lowrank_pair(uacc[j][2 * hr], uacc[j][2 * hr + 1], cs2, s.lr_rope, Act{s.lr_act});
+                        const float2 y = feature(uacc[j][2 * hr], uacc[j][2 * hr + 1], cs2);
                         zacc[j][0] += y.x;
                         zacc[j][1] += y.y;
                         asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(ktb + tl * C::KT + (nt * 8 + t4 * 2) * 2),
@@ -493,15 +510,15 @@ __global__ void prepass_combine_kernel(Shape s, int ctas, int units, const float
     }
 }
 
-template <int R, typename Act>
+template <int R, typename Feature>
 cudaError_t launch_ra(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const Params& p, int ctas,
                       bool fuse, cudaStream_t st)
 {
     const Layout lay(R, fuse);
-    cudaError_t e = cudaFuncSetAttribute(prepass_kernel<R, Act>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(prepass_kernel<R, Feature>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)lay.total);
     if (e != cudaSuccess) return e;
-    launch_kernel(prepass_kernel<R, Act>, ctas, kThreads, lay.total, st, mq, mk, mv, p);
+    launch_kernel(prepass_kernel<R, Feature>, ctas, kThreads, lay.total, st, mq, mk, mv, p);
     return cudaGetLastError();
 }
 
@@ -509,8 +526,8 @@ template <int R>
 cudaError_t launch_r(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const Params& p, int ctas,
                      bool fuse, cudaStream_t st)
 {
-    return p.s.lr_act == ROLA_LOWRANK_ACT_SILU ? launch_ra<R, SiluFast>(mq, mk, mv, p, ctas, fuse, st)
-                                               : launch_ra<R, ActAblation>(mq, mk, mv, p, ctas, fuse, st);
+    return default_feature(p.s) ? launch_ra<R, SiluOutside>(mq, mk, mv, p, ctas, fuse, st)
+                                : launch_ra<R, AnyFeature>(mq, mk, mv, p, ctas, fuse, st);
 }
 
 }  // namespace

@@ -62,14 +62,7 @@ struct Params {
     int splits;               // > 0: CTAs per head, none of which meets two heads
 };
 
-// SiLU with the MUFU exponential; the kernel is instantiated for it and for
-// ActAblation (the other feature maps of the activation ablation).
-struct SiluMufu {
-    int kind;    // always ROLA_LOWRANK_ACT_SILU
-    __device__ float operator()(float x) const { return silu(x); }
-};
-
-template <int R, typename Act>
+template <int R, typename Feature>
 __global__ void __launch_bounds__(32 * Layout<R>::warps, 1) readout_kernel(const __grid_constant__ CUtensorMap map_q,
                                                                           const __grid_constant__ CUtensorMap map_os,
                                                                           const __grid_constant__ CUtensorMap map_o,
@@ -97,6 +90,8 @@ __global__ void __launch_bounds__(32 * Layout<R>::warps, 1) readout_kernel(const
         u1 = (long long)bh * p.tiles + (long long)(i + 1) * p.tiles / p.splits;
     }
     const int hw = s.Hh * s.Ww;
+    const Feature feature(s);
+    const float2* tab = p.tab + t4;
 
     if (tid == 0) {
         *abort = 0;
@@ -191,16 +186,22 @@ __global__ void __launch_bounds__(32 * Layout<R>::warps, 1) readout_kernel(const
             // ---- q~: an accumulator's two rows and column pair are the A fragment of the next product
             // (rows of tokens past N are never stored)
             uint32_t af[R / 8][2];
+            auto features = [&](auto row) {              // row(pair, token): the pair's table row
 #pragma unroll
-            for (int j = 0; j < R / 8; ++j)
+                for (int j = 0; j < R / 8; ++j)
 #pragma unroll
-                for (int hr = 0; hr < 2; ++hr) {
-                    const int m = j * 4 + t4;
-                    const int row = m < s.pt ? tt[hr] : (m < s.pt + s.px ? s.T + xx[hr] : s.T + s.Hh + yy[hr]);
-                    const float2 f = lowrank_pair(u[j][2 * hr], u[j][2 * hr + 1], __ldg(p.tab + row * kPairs + m),
-                                                  s.lr_rope, Act{s.lr_act});
-                    af[j][hr] = pack_bf16(f.x, f.y);
-                }
+                    for (int hr = 0; hr < 2; ++hr) {
+                        const float2 f = feature(u[j][2 * hr], u[j][2 * hr + 1],
+                                                 __ldg(tab + row(j * 4 + t4, hr) * kPairs + j * 4));
+                        af[j][hr] = pack_bf16(f.x, f.y);
+                    }
+            };
+            // (with every pair on the temporal axis, r <= 44 by default, a token has one table row)
+            if (R / 2 <= s.pt) features([&](int, int hr) { return tt[hr]; });
+            else
+                features([&](int m, int hr) {
+                    return m < s.pt ? tt[hr] : (m < s.pt + s.px ? s.T + xx[hr] : s.T + s.Hh + yy[hr]);
+                });
             // ---- y = q~ C
             float y[16][4];
 #pragma unroll
@@ -218,36 +219,44 @@ __global__ void __launch_bounds__(32 * Layout<R>::warps, 1) readout_kernel(const
             ok = __all_sync(0xffffffffu, mbar_wait(o_full + 8 * buf, (i / OB) & 1, abort, s.wait_limit_ns));
             if (!ok) break;
             const uint32_t ob = qb + kBox + buf * kBox;
-            auto os = [&](int d, int hr) {               // this thread's pair of O^s (read twice: registers are short)
-                uint32_t w;
-                asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(w) : "r"(ob + wsw(g + 8 * hr, d) + t4 * 4));
-                return unpack_bf16(w);
-            };
+            // O^s in the accumulators' layout: the column pairs of two n-tiles, rows g and g + 8
+            // (read twice: y leaves no registers to keep it)
+            uint32_t w[2][2];
+            const uint32_t oaddr = (lane & 7) + (mi & 1) * 8;            // row this lane addresses
             float ssy[2] = {0.0f, 0.0f}, sso[2] = {0.0f, 0.0f};
 #pragma unroll
-            for (int d = 0; d < 16; ++d) {
+            for (int d = 0; d < 16; d += 2) {
+                ldsm_x4(ob + wsw(oaddr, d + (mi >> 1)), w[0][0], w[0][1], w[1][0], w[1][1]);
 #pragma unroll
-                for (int hr = 0; hr < 2; ++hr) {
-                    const float2 f = os(d, hr);
-                    ssy[hr] += y[d][2 * hr] * y[d][2 * hr] + y[d][2 * hr + 1] * y[d][2 * hr + 1];
-                    sso[hr] += f.x * f.x + f.y * f.y;
-                }
+                for (int e = d; e < d + 2; ++e)
+#pragma unroll
+                    for (int hr = 0; hr < 2; ++hr) {
+                        const float2 f = unpack_bf16(w[e - d][hr]);
+                        ssy[hr] += y[e][2 * hr] * y[e][2 * hr] + y[e][2 * hr + 1] * y[e][2 * hr + 1];
+                        sso[hr] += f.x * f.x + f.y * f.y;
+                    }
             }
+            float coef[2];
 #pragma unroll
             for (int hr = 0; hr < 2; ++hr) {
                 ssy[hr] += __shfl_xor_sync(0xffffffffu, ssy[hr], 1);
                 ssy[hr] += __shfl_xor_sync(0xffffffffu, ssy[hr], 2);
                 sso[hr] += __shfl_xor_sync(0xffffffffu, sso[hr], 1);
                 sso[hr] += __shfl_xor_sync(0xffffffffu, sso[hr], 2);
-                const float coef = gp[hr] * sqrtf(sso[hr] * (1.0f / kDh) + s.eps_fuse) *
-                                   rsqrtf(ssy[hr] * (1.0f / kDh) + s.eps_lr);
+                coef[hr] = gp[hr] * sqrtf(sso[hr] * (1.0f / kDh) + s.eps_fuse) *
+                           rsqrtf(ssy[hr] * (1.0f / kDh) + s.eps_lr);
+            }
 #pragma unroll
-                for (int d = 0; d < 16; ++d) {
-                    const float2 f = os(d, hr);
-                    asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(ob + wsw(g + 8 * hr, d) + t4 * 4),
-                                 "r"(pack_bf16(f.x + coef * y[d][2 * hr], f.y + coef * y[d][2 * hr + 1]))
-                                 : "memory");
-                }
+            for (int d = 0; d < 16; d += 2) {
+                ldsm_x4(ob + wsw(oaddr, d + (mi >> 1)), w[0][0], w[0][1], w[1][0], w[1][1]);
+#pragma unroll
+                for (int e = d; e < d + 2; ++e)
+#pragma unroll
+                    for (int hr = 0; hr < 2; ++hr) {
+                        const float2 f = unpack_bf16(w[e - d][hr]);
+                        w[e - d][hr] = pack_bf16(f.x + coef[hr] * y[e][2 * hr], f.y + coef[hr] * y[e][2 * hr + 1]);
+                    }
+                stsm_x4(ob + wsw(oaddr, d + (mi >> 1)), w[0][0], w[0][1], w[1][0], w[1][1]);
             }
             fence_proxy_async_smem();
             __syncwarp();
@@ -271,16 +280,16 @@ __global__ void __launch_bounds__(32 * Layout<R>::warps, 1) readout_kernel(const
     }
 }
 
-template <int R, typename Act>
+template <int R, typename Feature>
 cudaError_t launch_ra(const CUtensorMap& mq, const CUtensorMap& mos, const CUtensorMap& mo, const Params& p, int ctas,
                       cudaStream_t st)
 {
     using L = Layout<R>;
     static_assert(L::total <= 232448, "fits the shared memory of one SM");
     cudaError_t e =
-        cudaFuncSetAttribute(readout_kernel<R, Act>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::total);
+        cudaFuncSetAttribute(readout_kernel<R, Feature>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::total);
     if (e != cudaSuccess) return e;
-    launch_kernel(readout_kernel<R, Act>, ctas, 32 * L::warps, L::total, st, mq, mos, mo, p);
+    launch_kernel(readout_kernel<R, Feature>, ctas, 32 * L::warps, L::total, st, mq, mos, mo, p);
     return cudaGetLastError();
 }
 
@@ -288,8 +297,8 @@ template <int R>
 cudaError_t launch_r(const CUtensorMap& mq, const CUtensorMap& mos, const CUtensorMap& mo, const Params& p, int ctas,
                      cudaStream_t st)
 {
-    return p.s.lr_act == ROLA_LOWRANK_ACT_SILU ? launch_ra<R, SiluMufu>(mq, mos, mo, p, ctas, st)
-                                               : launch_ra<R, ActAblation>(mq, mos, mo, p, ctas, st);
+    return default_feature(p.s) ? launch_ra<R, SiluOutside>(mq, mos, mo, p, ctas, st)
+                                : launch_ra<R, AnyFeature>(mq, mos, mo, p, ctas, st);
 }
 
 }  // namespace
