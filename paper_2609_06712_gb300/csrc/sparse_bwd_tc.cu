@@ -18,13 +18,16 @@
 // products, so neither passes through shared memory.  The log-sum-exp of each
 // query is known, so a tile needs no running maximum: eight warps share it, a
 // thread 32 columns of one row (warpgroup w: block w of the pair; the two half
-// warps 32 columns each).  One thread issues every product, in an order that
-// leaves each result two products' time (about 1000 cycles) until it is needed
-// again, so S, dP and the accumulators are single-buffered:
-//   query side: S(g+1) dP(g+1) dQ(g)             dS double-buffered
-//   key side:   S(g+1) dK(g) dP(g+1) dV(g+1)     P written over S, dS over dP
-//     (products of one thread run in order, so S(g+1) may overwrite the P(g)
-//     that dV(g) read)
+// warps 32 columns each).  Each result has one or two products' time (512 cycles
+// each) until it is needed again, so S, dP and the accumulators are single-buffered.
+//   query side: S, dP of a tile by one thread, dQ by another     dS double-buffered
+//     (an issuer spends 75 cycles on every barrier it waits for even when that is
+//     complete, and the pipe runs dry meanwhile: one thread for all took 18.1 ms
+//     where this takes 16.0, 720p layer)
+//   key side:   S(g+1) dK(g) dP(g+1) dV(g+1) by one thread       P written over S, dS over dP
+//     (products of one thread run in order, so S(g+1) may overwrite the P(g) that
+//     dV(g) read; with S, dV and dP, dK on two threads the order drifts, and the
+//     kernel took 25.7 ms instead of 21.6)
 //
 // What bounds it: an M = 64, N = 128 product takes 64 cycles a K step of 16 (half
 // the M = 128 rate), 1536 (query side) and 2048 (key side) tensor cycles a
@@ -33,15 +36,15 @@
 // and 1536 tensor cycles, P and dS through shared memory) moved 224 and 288 KB,
 // and its two-deep rings of 64 KB pairs were held through the whole tile.  At
 // the 720p layer (40 heads, 75600 tokens, 118 of 1182 blocks kept): query side
-// 27.3 -> 18.2 ms, key side 37.9 -> 21.9 ms (992 / 1192 ns a tile; the products
-// alone take 845 / 1126 ns at the 1.82 GHz the SMs hold under this load); at
-// the 12-head 480p layer 1.84 -> 1.12 and 2.52 -> 1.40 ms.
+// 27.3 -> 16.0 ms, key side 37.9 -> 21.9 ms (872 / 1192 ns a tile; the products
+// alone take 750 / 1000 ns at the 2.05 GHz the SMs hold under this load); at
+// the 12-head 480p layer 1.84 -> 0.99 and 2.52 -> 1.40 ms.
 //
 // Roles (384 threads, one persistent CTA per SM):
 //   warps 0-7  P / dS and the epilogue; warp w owns TMEM lane quarter w mod 4
 //   warps 8, 9 TMA producers (one elected thread each)
-//   warp 10    issuer of every product, TMEM owner
-//   warp 11    key side: log-sum-exp and D of a tile's queries into shared memory
+//   warp 10    issuer and TMEM owner
+//   warp 11    query side: second issuer; key side: log-sum-exp and D of a tile's queries into shared memory
 // Every mbarrier wait is bounded; a wait that gives up records ROLA_ERR_TIMEOUT
 // and the CTA drains what it issued and frees TMEM.
 #include <math_constants.h>
@@ -58,7 +61,7 @@ using namespace tc;
 
 constexpr int kDsWarps = 8;
 constexpr int kCols = 32;                        // tile columns of a dS thread
-constexpr int kProdAWarp = 8, kProdBWarp = 9, kMmaWarp = 10, kStatWarp = 11;
+constexpr int kProdAWarp = 8, kProdBWarp = 9, kMmaWarp = 10, kMma2Warp = 11, kStatWarp = 11;
 constexpr int kThreads = 32 * 12;
 constexpr uint32_t kBlockBytes = 64 * 128 * 2;   // one block, [chunk][row][64]
 constexpr uint32_t kPairBytes = 128 * 128 * 2;   // a pair of blocks, [chunk][block][row][64]
@@ -141,6 +144,9 @@ __device__ __forceinline__ void mma_grad(uint32_t d, uint32_t a, uint32_t gap, u
     for (int kk = 0; kk < 4; ++kk) mma_ts_split(d, a + gap + kk * 8, b + (kk + 4) * 128, b_hi, id, 1u);
 }
 
+// The 128 bytes at p into L2 (the epilogue's rows, asked for when the item starts).
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p)); }
+
 // The 32 outputs of a thread (columns d0 .. d0 + 31 of one row) at dst, as bf16.
 __device__ __forceinline__ void store_row32(__nv_bfloat16* dst, const float (&v)[kCols])
 {
@@ -194,7 +200,7 @@ constexpr uint32_t kS = 0, kDP = 128, kDQ = 256, kDS = 384;     // TMEM columns 
 
 enum Bar { Q_FULL = 0, Q_EMPTY = Q_FULL + 2, K_FULL = Q_EMPTY + 2, K_EMPTY = K_FULL + KS, V_FULL = K_EMPTY + KS,
            V_EMPTY = V_FULL + VS, S_FULL = V_EMPTY + VS, S_EMPTY, DP_FULL, DP_EMPTY, DS_FULL, DS_EMPTY = DS_FULL + 2,
-           O_FULL = DS_EMPTY + 2, O_EMPTY, DRAIN, NUM_BARS };
+           O_FULL = DS_EMPTY + 2, O_EMPTY, DRAIN, NUM_BARS = DRAIN + 2 };
 
 struct Ctrl {
     uint64_t bar[NUM_BARS];
@@ -296,33 +302,34 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
             for (int u = issued > NS ? issued - NS : 0; u < issued; ++u)
                 mbar_wait(bar(full0 + u % NS), (u / NS) & 1, &never, s.wait_limit_ns);
         }
-    } else if (warp == kMmaWarp) {
-        // ------------------------------------------------------------ S(g), dP(g), dQ(g - 1), tile by tile
+    } else if (warp == kMmaWarp || warp == kMma2Warp) {
+        // ------------------------------------------------------------ issuers: S and dP / dQ
         if (elect_one()) {
+            const bool grad = warp == kMma2Warp;
             const uint32_t id_s = idesc_bf16(64, 128, false, false), id_g = idesc_bf16(64, 128, false, true);
             const uint64_t dk = smem_desc(sbase, 16, 1024);          // K-major operands
             const uint64_t dm = smem_desc(sbase, 16384, 1024);       // a pair read MN-major (chunks 16 KB apart)
             const uint32_t lo = (uint32_t)dk, hi = (uint32_t)(dk >> 32), mlo = (uint32_t)dm, mhi = (uint32_t)(dm >> 32);
             bool ok = true;
             int k = 0, g = 0;
-            // dQ += dS K of tile u, the t-th of item ku
-            auto grad = [&](int u, int t, int ku) -> bool {
-                if (t == 0 && ku >= 1 && !mbar_wait(bar(O_EMPTY), (ku - 1) & 1, abort, s.wait_limit_ns)) return false;
-                if (!mbar_wait(bar(DS_FULL + (u & 1)), (u >> 1) & 1, abort, s.wait_limit_ns)) return false;
-                fence_after_sync();
-                const uint32_t b = mlo + ((kSmK + (u % KS) * kPairBytes) >> 4);
-                mma_grad(tmem + kDQ, tmem + kDS + (u & 1) * 64, 32, b, mhi, id_g, 2 * t + 1 >= s.n_keep, t == 0);
-                mma_commit(bar(DS_EMPTY + (u & 1)));
-                mma_commit(bar(K_EMPTY + u % KS));
-                if (t == T - 1) mma_commit(bar(O_FULL));
-                return true;
-            };
             for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x, ++k) {
                 const int qs = k & 1;
-                if (!(ok = mbar_wait(bar(Q_FULL + qs), (k >> 1) & 1, abort, s.wait_limit_ns))) break;
+                if (!grad && !(ok = mbar_wait(bar(Q_FULL + qs), (k >> 1) & 1, abort, s.wait_limit_ns))) break;
                 const uint32_t q = lo + ((kSmQ + qs * kBlockBytes) >> 4), o = lo + ((kSmO + qs * kBlockBytes) >> 4);
                 for (int t = 0; t < T; ++t, ++g) {
-                    const int ks = g % KS, vs = g % VS;
+                    const int ks = g % KS, vs = g % VS, db = g & 1;
+                    if (grad) {
+                        if (!(ok = mbar_wait(bar(K_FULL + ks), (g / KS) & 1, abort, s.wait_limit_ns))) break;
+                        if (t == 0 && k >= 1 && !(ok = mbar_wait(bar(O_EMPTY), (k - 1) & 1, abort, s.wait_limit_ns))) break;
+                        if (!(ok = mbar_wait(bar(DS_FULL + db), (g >> 1) & 1, abort, s.wait_limit_ns))) break;
+                        fence_after_sync();
+                        mma_grad(tmem + kDQ, tmem + kDS + db * 64, 32, mlo + ((kSmK + ks * kPairBytes) >> 4), mhi, id_g,
+                                 2 * t + 1 >= s.n_keep, t == 0);
+                        mma_commit(bar(DS_EMPTY + db));
+                        mma_commit(bar(K_EMPTY + ks));
+                        if (t == T - 1) mma_commit(bar(O_FULL));
+                        continue;
+                    }
                     if (!(ok = mbar_wait(bar(K_FULL + ks), (g / KS) & 1, abort, s.wait_limit_ns))) break;
                     if (g >= 1 && !(ok = mbar_wait(bar(S_EMPTY), (g - 1) & 1, abort, s.wait_limit_ns))) break;
                     fence_after_sync();
@@ -335,15 +342,13 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
                     mma_commit(bar(DP_FULL));
                     mma_commit(bar(V_EMPTY + vs));
                     if (t == T - 1) mma_commit(bar(Q_EMPTY + qs));
-                    if (g >= 1 && !(ok = t > 0 ? grad(g - 1, t - 1, k) : grad(g - 1, T - 1, k - 1))) break;
                 }
             }
-            if (ok && g > 0) ok = grad(g - 1, T - 1, k - 1);
-            if (!ok) record_timeout(p, 18);
+            if (!ok) record_timeout(p, grad ? 21 : 18);
             // every product this thread issued completes before TMEM is released
             int never = 0;
-            mma_commit(bar(DRAIN));
-            mbar_wait(bar(DRAIN), 0, &never, s.wait_limit_ns);
+            mma_commit(bar(DRAIN + grad));
+            mbar_wait(bar(DRAIN + grad), 0, &never, s.wait_limit_ns);
         }
     } else if (warp < kDsWarps) {
         // ------------------------------------------------------------ dS + epilogue
@@ -360,6 +365,8 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
             const size_t r = (size_t)bh * s.Np + (size_t)qb * 64 + row;
             const float l2 = n >= 0 ? __ldg(p.lse + r) * kLog2e : CUDART_INF_F;
             const float Dn = n >= 0 ? -__ldg(p.Dv + r) : 0.0f;
+            const size_t at = ((size_t)bh * s.N + (n >= 0 ? n : 0)) * kDh + d0;
+            prefetch_l2(p.lr0 + at);                                    // this thread's row part of the epilogue
             int j_n = wg < s.n_keep ? __ldg(kept + wg) : -1;            // this group's block, one tile ahead
             for (int t = 0; t < T; ++t, ++g) {
                 const int j = j_n;
@@ -406,7 +413,6 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
             // of its row.  What does not depend on dQ is read before the wait for it.
             float lr[kCols], v[kCols];
             float2 cs[16];
-            const size_t at = ((size_t)bh * s.N + (n >= 0 ? n : 0)) * kDh + d0;
             load_row32(p.lr0 + at, lr);
             load_cs(p, n >= 0 ? n : 0, d0, cs);
             if (!(ok = mbar_wait(bar(O_FULL), k & 1, abort, s.wait_limit_ns))) break;
@@ -662,6 +668,9 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
             range(item, bh, kb, len);
             const int T = (len + 1) / 2;
             const int n = slot_token_g<kCube>(s, kb, row);            // this row's token, -1 for an empty slot
+            const size_t at = ((size_t)bh * s.N + (n >= 0 ? n : 0)) * kDh + d0;
+            prefetch_l2(p.lr0 + at);                                   // this thread's row parts of the epilogue
+            prefetch_l2(p.lr1 + at);
             for (int t = 0; t < T; ++t, ++g) {
                 float x[kCols], y[kCols];
                 if (!(ok = mbar_wait(bar(Q_FULL + g % QS), (g / QS) & 1, abort, s.wait_limit_ns))) break;   // lse, D are there
@@ -700,17 +709,14 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
             // ---- epilogue: dk = low-rank row + R(p)^T (dK / sqrt d), dv = low-rank row + dV; this
             // thread's 32 columns of its row.  A key block no query block kept has the low-rank
             // rows alone.
-            float lr[kCols], v[kCols];
+            float lr[kCols], v[kCols], w[kCols];
             float2 cs[16];
-            const size_t at = ((size_t)bh * s.N + (n >= 0 ? n : 0)) * kDh + d0;
             load_row32(p.lr1 + at, lr);
             load_cs(p, n >= 0 ? n : 0, d0, cs);
             if (len > 0) {
                 if (!(ok = mbar_wait(bar(ACC_FULL), k & 1, abort, s.wait_limit_ns))) break;
                 fence_after_sync();
-                ld_cols(base + kDV + 64 * wg, v);
-#pragma unroll
-                for (int i = 0; i < kCols; ++i) lr[i] += v[i];
+                ld_cols(base + kDV + 64 * wg, w);
                 ld_cols(base + kDK + 64 * wg, v);
                 fence_before_sync();
                 __syncwarp();
@@ -718,9 +724,11 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
                 ++k;
             } else {
 #pragma unroll
-                for (int i = 0; i < kCols; ++i) v[i] = 0.0f;
+                for (int i = 0; i < kCols; ++i) v[i] = w[i] = 0.0f;
             }
             if (n >= 0) {
+#pragma unroll
+                for (int i = 0; i < kCols; ++i) lr[i] += w[i];
                 store_row32(p.out1 + at, lr);
                 load_row32(p.lr0 + at, lr);
                 rotate_back32(v, lr, cs);
