@@ -26,8 +26,11 @@ constexpr int kPairs = kDh / 2;
 struct DeviceStatus {
     int32_t code;             // rola_status_t of the last failing device-side check
     int32_t where;            // kernel-specific site id
-    int32_t pad[62];
+    int32_t next[4];          // items handed out so far by the persistent kernels of a call (ItemCounter)
+    int32_t pad[58];
 };
+// Which counter a persistent kernel takes its items from; all are zero when a call's kernels start.
+enum ItemCounter { kItemsForward = 0, kItemsDq = 1, kItemsDkDv = 2 };
 
 // Kernel-side view of a validated configuration.
 struct Shape {

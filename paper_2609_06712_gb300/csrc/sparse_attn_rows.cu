@@ -120,6 +120,7 @@ struct Ctrl {
     float m[2][QN];                      // -m of every row after an even / odd tile
     float2 l[2][QN];                     // (row sum, its -m) of the group that does not end item k, by k & 1
     uint64_t bar[Cfg<QN>::NUM_BARS];
+    ItemRing items;
     uint32_t tmem_base;
     int abort;
 };
@@ -232,6 +233,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
             mbar_init(bar(L_READY + i), 1);
         }
         mbar_init(bar(O_EMPTY), kWarpsPerGroup);
+        sm.items.init();
         fence_mbar_init();
     }
     if (warp == kMmaWarp) {
@@ -249,6 +251,9 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
     const uint32_t tmem = sm.tmem_base;
     chain_begin();
     volatile int* abort = &sm.abort;
+    // the CTA's i-th item, for a single-thread role and for a warp
+    auto item_at = [&](int i, bool& ok) { return sm.items.get<true>(i, ok, abort, s.wait_limit_ns); };
+    auto item_at_warp = [&](int i, bool& ok) { return sm.items.get<false>(i, ok, abort, s.wait_limit_ns); };
 
     if constexpr (QN == 128) {
         if (warp >= kProducerKWarp) regs_dec<88>();    // the softmax groups take 208: 208 + 208 + 88 = 3 x 168
@@ -263,7 +268,14 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
         if (elect_one()) {
             int k = 0, g = 0, issued_q = 0, issued = 0;
             bool ok = true;
-            for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x, ++k) {
+            // (the K warp hands out the items: the next one is known, the one after asked for)
+            int item = is_v ? item_at(0, ok) : (int)blockIdx.x, next = 0;
+            int* counter = &p.status->next[kItemsForward];
+            if (!is_v) {
+                sm.items.post(0, item, abort, s.wait_limit_ns);
+                next = gridDim.x + atomicAdd(counter, 1);
+            }
+            for (; item < p.total_items && ok; ++k) {
                 const int bh = item / nI, qb = item - bh * nI;
                 const int32_t* kept = p.kv_idx + (size_t)item * s.n_keep;
                 int ja_n = __ldg(kept), jb_n = s.n_keep > 1 ? __ldg(kept + 1) : -1;     // block ids, one tile ahead
@@ -275,7 +287,13 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
                     tma_load_4d(sbase + kSmemQ + qs * kQBytes, &map_q, bar(Q_FULL + qs), 0, qb * QN, 0, bh);
                     ++issued_q;
                 }
+                int after = 0;
                 for (int t = 0; t < T; ++t, ++g) {
+                    // (the first answer of the counter is given time: it is not needed before the second tile)
+                    if (!is_v && t == (k == 0 && T > 1 ? 1 : 0)) {
+                        if (!(ok = sm.items.post(k + 1, next, abort, s.wait_limit_ns))) break;
+                        after = gridDim.x + atomicAdd(counter, 1);
+                    }
                     const int ra = ja_n * 64, rb = jb_n * 64;
                     const bool two = jb_n >= 0;                 // the last tile of an odd n_keep holds one block
                     if (t + 1 < T) {
@@ -314,6 +332,9 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
                         }
                     }
                 }
+                if (!ok) break;
+                if (is_v) item = item_at(k + 1, ok);
+                else item = next, next = after;
             }
             if (!ok) record_timeout(p, is_v ? 4 : 1);
             // every copy this thread issued lands before the CTA exits (bounded by time only)
@@ -339,7 +360,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
             const uint32_t v_lo = (uint32_t)dv, v_hi = (uint32_t)(dv >> 32);
             bool ok = true;
             int k = 0;
-            for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x, ++k) {
+            for (int item = item_at(0, ok); item < p.total_items && ok; item = item_at(++k, ok)) {
                 if (!pv) {
                     const int qs = k % QB;
                     if (!(ok = mbar_wait(bar(Q_FULL + qs), (k / QB) & 1, abort, s.wait_limit_ns))) break;
@@ -416,7 +437,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_attn_rows_kernel(const __g
                        o_addr = tmem + lane_off + kTmemO;
         bool ok = true;
         int k = 0;
-        for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x, ++k) {
+        for (int item = item_at_warp(0, ok); item < p.total_items && ok; item = item_at_warp(++k, ok)) {
             const int bh = item / nI, qb = item - bh * nI;
             const int32_t* kept = p.kv_idx + (size_t)item * s.n_keep;
             const int g0 = k * T;

@@ -204,6 +204,7 @@ enum Bar { Q_FULL = 0, Q_EMPTY = Q_FULL + 2, K_FULL = Q_EMPTY + 2, K_EMPTY = K_F
 
 struct Ctrl {
     uint64_t bar[NUM_BARS];
+    ItemRing items;
     uint32_t tmem_base;
     int abort;
 };
@@ -237,6 +238,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
             const bool by_warps = i == S_EMPTY || i == DP_EMPTY || i == DS_FULL || i == DS_FULL + 1 || i == O_EMPTY;
             mbar_init(bar(i), by_warps ? kDsWarps : 1);
         }
+        sm.items.init();
         fence_mbar_init();
     }
     if (warp == kMmaWarp) {
@@ -255,6 +257,9 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
     const uint32_t tmem = sm.tmem_base;
     chain_begin();
     volatile int* abort = &sm.abort;
+    // the CTA's i-th item, for a single-thread role and for a warp
+    auto item_at = [&](int i, bool& ok) { return sm.items.get<true>(i, ok, abort, s.wait_limit_ns); };
+    auto item_at_warp = [&](int i, bool& ok) { return sm.items.get<false>(i, ok, abort, s.wait_limit_ns); };
 
     if (warp == kProdAWarp || warp == kProdBWarp) {
         // ------------------------------------------------------------ TMA: Q, dO and the K pairs / the V pairs
@@ -266,7 +271,14 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
         if (elect_one()) {
             int k = 0, issued_q = 0, issued = 0;
             bool ok = true;
-            for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x, ++k) {
+            // (the K warp hands out the items: the next one is known, the one after asked for)
+            int item = is_v ? item_at(0, ok) : (int)blockIdx.x, next = 0;
+            int* counter = &p.status->next[kItemsDq];
+            if (!is_v) {
+                sm.items.post(0, item, abort, s.wait_limit_ns);
+                next = gridDim.x + atomicAdd(counter, 1);
+            }
+            for (; item < p.total_items && ok; ++k) {
                 const int bh = item / nB, qb = item - bh * nB;
                 const int32_t* kept = p.kv_idx + (size_t)item * s.n_keep;
                 int ja_n = __ldg(kept), jb_n = s.n_keep > 1 ? __ldg(kept + 1) : -1;     // block ids, one tile ahead
@@ -278,7 +290,13 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
                     tma_load_4d(sbase + kSmO + qs * kBlockBytes, &map_o, bar(Q_FULL + qs), 0, qb * 64, 0, bh);
                     ++issued_q;
                 }
+                int after = 0;
                 for (int t = 0; t < T; ++t) {
+                    // (the first answer of the counter is given time: it is not needed before the second tile)
+                    if (!is_v && t == (k == 0 && T > 1 ? 1 : 0)) {
+                        if (!(ok = sm.items.post(k + 1, next, abort, s.wait_limit_ns))) break;
+                        after = gridDim.x + atomicAdd(counter, 1);
+                    }
                     const int g = issued, st = g % NS;
                     const int ra = ja_n * 64, rb = jb_n * 64;
                     const bool two = jb_n >= 0;
@@ -293,6 +311,9 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
                     mbar_expect_tx(bar(full0 + st), two ? 32768u : 16384u);
                     load_pair(sbase + ring + st * kPairBytes, map, bar(full0 + st), ra, rb, two, bh);
                 }
+                if (!ok) break;
+                if (is_v) item = item_at(k + 1, ok);
+                else item = next, next = after;
             }
             if (!ok) record_timeout(p, is_v ? 20 : 17);
             // every copy this thread issued lands before the CTA exits (bounded by time only)
@@ -312,7 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
             const uint32_t lo = (uint32_t)dk, hi = (uint32_t)(dk >> 32), mlo = (uint32_t)dm, mhi = (uint32_t)(dm >> 32);
             bool ok = true;
             int k = 0, g = 0;
-            for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x, ++k) {
+            for (int item = item_at(0, ok); item < p.total_items && ok; item = item_at(++k, ok)) {
                 const int qs = k & 1;
                 if (!grad && !(ok = mbar_wait(bar(Q_FULL + qs), (k >> 1) & 1, abort, s.wait_limit_ns))) break;
                 const uint32_t q = lo + ((kSmQ + qs * kBlockBytes) >> 4), o = lo + ((kSmO + qs * kBlockBytes) >> 4);
@@ -358,7 +379,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
         const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16);
         bool ok = true;
         int k = 0, g = 0;
-        for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x, ++k) {
+        for (int item = item_at_warp(0, ok); item < p.total_items && ok; item = item_at_warp(++k, ok)) {
             const int bh = item / nB, qb = item - bh * nB;
             const int32_t* kept = p.kv_idx + (size_t)item * s.n_keep;
             const int n = slot_token_g<kCube>(s, qb, row);             // this row's token, -1 for an empty slot
@@ -448,6 +469,7 @@ struct Ctrl {
     float lse2[2][128];                  // log-sum-exp (log2 units) and -D of an even / odd tile's queries
     float nD[2][128];
     uint64_t bar[NUM_BARS];
+    ItemRing items;
     uint32_t tmem_base;
     int abort;
 };
@@ -491,6 +513,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
             const bool q_full = i >= Q_FULL && i < Q_FULL + QS;       // the Q pair and the tile's lse, D
             mbar_init(bar(i), by_warps ? kDsWarps : (q_full ? 2 : 1));
         }
+        sm.items.init();
         fence_mbar_init();
     }
     if (warp == kMmaWarp) {
@@ -509,6 +532,9 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
     const uint32_t tmem = sm.tmem_base;
     chain_begin();
     volatile int* abort = &sm.abort;
+    // the CTA's i-th item, for a single-thread role and for a warp
+    auto item_at = [&](int i, bool& ok) { return sm.items.get<true>(i, ok, abort, s.wait_limit_ns); };
+    auto item_at_warp = [&](int i, bool& ok) { return sm.items.get<false>(i, ok, abort, s.wait_limit_ns); };
 
     if (warp == kProdAWarp || warp == kProdBWarp) {
         // ------------------------------------------------------------ TMA: K, V and the Q pairs / the dO pairs
@@ -520,7 +546,26 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
         if (elect_one()) {
             int k = 0, issued_kv = 0, issued = 0;
             bool ok = true;
-            for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x) {
+            // (the Q warp hands out the items: the next one is known, the one after asked for; i counts
+            // them, k those that some query block kept)
+            int next = 0, after = 0;
+            int* counter = &p.status->next[kItemsDkDv];
+            if (!is_o) {
+                sm.items.post(0, blockIdx.x, abort, s.wait_limit_ns);
+                next = gridDim.x + atomicAdd(counter, 1);
+            }
+            auto advance = [&](int i) {                       // the item after the i-th
+                if (is_o) return item_at(i + 1, ok);
+                const int x = next;
+                next = after;
+                return x;
+            };
+            int i = 0;
+            for (int item = is_o ? item_at(0, ok) : (int)blockIdx.x; item < p.total_items && ok; item = advance(i), ++i) {
+                if (!is_o) {
+                    if (!(ok = sm.items.post(i + 1, next, abort, s.wait_limit_ns))) break;
+                    after = gridDim.x + atomicAdd(counter, 1);
+                }
                 int bh, kb, len;
                 const int32_t* l = range(item, bh, kb, len);
                 if (len == 0) continue;
@@ -565,7 +610,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
         // block: lse = +inf, so its P is 0); read one tile ahead
         int g = 0;
         bool ok = true;
-        for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x) {
+        for (int it = 0, item = item_at_warp(0, ok); item < p.total_items && ok; item = item_at_warp(++it, ok)) {
             int bh, kb, len;
             const int32_t* l = range(item, bh, kb, len);
             const int T = (len + 1) / 2;
@@ -616,7 +661,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
                 if (last) mma_commit(bar(ACC_FULL));
                 return true;
             };
-            for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x) {
+            for (int i = 0, item = item_at(0, ok); item < p.total_items && ok; item = item_at(++i, ok)) {
                 int bh, kb, len;
                 range(item, bh, kb, len);
                 if (len == 0) continue;
@@ -663,7 +708,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
         const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16);
         bool ok = true;
         int k = 0, g = 0;
-        for (int item = blockIdx.x; item < p.total_items && ok; item += gridDim.x) {
+        for (int i = 0, item = item_at_warp(0, ok); item < p.total_items && ok; item = item_at_warp(++i, ok)) {
             int bh, kb, len;
             range(item, bh, kb, len);
             const int T = (len + 1) / 2;
