@@ -63,16 +63,17 @@
 //   - two softmax groups in turn: 11.85 -> 11.5 ms (QN = 64), 8.2 -> 7.3 ms (QN = 128).
 //   - cube blocks on this kernel instead of a transposed form of their own: 4.88 ->
 //     3.43 ms (40 heads, 21 x 30 x 52 grid, 62 of 624 cubes kept).
-//   - QN = 64 now takes 1137 cycles a tile: 1024 of tensor work (an M = 64
-//     product runs at half the M = 128 rate) and 144 KB through the shared
-//     memory (1125 at 128 B/cycle).  QN = 128 takes ~1400 cycles against the
-//     same 1024, its softmax groups 2350 of the 2800 cycles they have.  The SM
-//     clock falls to 1.73-1.82 GHz (from 2.07) under the denser kernels.
+//   - items off a counter instead of dealt out evenly: 11.5 -> 11.2 ms (QN = 64).
+//   - QN = 64 takes ~1240 cycles a tile: 1024 of tensor work (an M = 64 product
+//     runs at half the M = 128 rate) and 144 KB through the shared memory (1125 at
+//     128 B/cycle).  QN = 128 takes ~1350 against the same 1024.  The 1400 W power
+//     cap sets the clock: 1.95-2.03 GHz for QN = 64, 1.72-1.82 GHz for QN = 128,
+//     whose 1650 TFLOP/s are 0.95 of the rate a GEMM sustains under that cap.
 //
 // Per 64-query block and 128-key tile the shared memory sees 64 KB of TMA
 // writes (K, V) and 80 KB of operand reads (Q 16, K 32, V 32) for 4.2 MFLOP,
-// against 176 KB in the transposed form of sparse_attn_tc.cu (which is kept
-// for the cube geometry); an M = 64 MMA runs at half the M = 128 rate.
+// against 176 KB in a transposed form (S^T with M = 128 keys, P^T through
+// shared memory); an M = 64 MMA runs at half the M = 128 rate.
 #include <cudaTypedefs.h>
 #include <stddef.h>
 

@@ -237,19 +237,8 @@ __device__ __forceinline__ void fence_after_sync()
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem]; issued by one thread.
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum)
-{
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
-        : "memory");
-}
-
-// As mma_ss, with each descriptor passed as (lo, hi) 32-bit halves so that a
-// K step only adds to lo (the start address field; no carry below 256 KB).
+// D[tmem] (+)= A[smem] * B[smem]; issued by one thread.  Each descriptor is passed as
+// (lo, hi) 32-bit halves so that a K step only adds to lo (the start address field; no carry below 256 KB).
 __device__ __forceinline__ void mma_ss_split(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
                                              uint32_t b_hi, uint32_t idesc, uint32_t accum)
 {
