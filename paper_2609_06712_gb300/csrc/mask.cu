@@ -5,6 +5,8 @@
 // pooled ROTATED vectors, s_ij = q_bar_i . k_bar_j / sqrt(d_h), keeps the
 // n_keep largest per row (ties to the lower block id) and lists them
 // ascending.  All score arithmetic is fp32.
+#include <float.h>
+
 #include "common.cuh"
 
 namespace rola {
@@ -121,9 +123,11 @@ __global__ void __launch_bounds__(256, 2) block_scores_kernel(Shape s, const flo
 // The threshold: a 256-bin histogram that is linear between the row's least and
 // largest score (a monotone map, so the counts give the bin of the n_keep-th
 // largest), then the handful of scores in that bin are ranked against each other.
-// Rows where that does not apply (a score that is not finite, a range too small to
-// divide, a bin with over 128 scores) take a 4-pass 8-bit radix select on
-// order-preserving keys.
+// Rows where that does not apply (a score that is not finite, all scores equal, a bin
+// with over 128 scores) take a 4-pass 8-bit radix select on order-preserving keys.
+// The map's shift is rounded, so where the scores differ by a few last bits only, the
+// whole row may land far below bin 0 or above bin 255; the end bins take those in, both
+// where scores are counted and where a bin's scores are listed.
 //
 // Bound by instruction issue: rows of 1182 took ~2600 instructions each with the
 // radix select, or with a loop that tests every element's index; so the registers
@@ -257,10 +261,11 @@ __global__ void __launch_bounds__(kTopkWarps * 32) block_topk_kernel(Shape s, co
         const int count = (int)hist[bin];
         __syncwarp();
         if (count <= 128) {
-            // the bin's scores and blocks, in block order, where the counts were (t in [t0, t1) is `bin`; -inf is outside)
+            // the bin's scores and blocks, in block order, where the counts were: t in [t0, t1) is the
+            // bin that LinearBins::bin gives (t of a score is finite, of the fill -inf: outside)
             float* cand = reinterpret_cast<float*>(hist);
             int* cand_j = reinterpret_cast<int*>(hist + 128);
-            const float t0 = bin == 0 ? -1.0f : (float)bin, t1 = bin == 255 ? INFINITY : (float)(bin + 1);
+            const float t0 = bin == 0 ? -FLT_MAX : (float)bin, t1 = bin == 255 ? INFINITY : (float)(bin + 1);
             int n = 0;
 #pragma unroll
             for (int i = 0; i < K; ++i) {
@@ -277,8 +282,8 @@ __global__ void __launch_bounds__(kTopkWarps * 32) block_topk_kernel(Shape s, co
                 }
             }
             __syncwarp();
-            pick(cand, cand_j, count, s.n_keep - above - 1, thr, last);
-            found = true;
+            found = n == count;
+            if (found) pick(cand, cand_j, count, s.n_keep - above - 1, thr, last);
         }
     }
     // word w: the kept blocks 32 w .. 32 w + 31; lane l takes words l and 32 + l
@@ -400,8 +405,8 @@ __global__ void __launch_bounds__(kTopkWarps * 32) block_topk_long_kernel(Shape 
                 n += __popc(m);
             }
             __syncwarp();
-            pick(cand, cand_j, count, s.n_keep - above - 1, thr, last);
-            found = true;
+            found = n == count;
+            if (found) pick(cand, cand_j, count, s.n_keep - above - 1, thr, last);
         }
     }
     uint32_t prefix = 0, pmask = 0;
