@@ -651,20 +651,29 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
             const uint32_t lo = (uint32_t)dk, hi = (uint32_t)(dk >> 32), mlo = (uint32_t)dm, mhi = (uint32_t)(dm >> 32);
             bool ok = true;
             int k = 0, g = 0;
-            bool prev_half = false, prev_first = false, prev_last = false;
-            // dK += dS^T Q of tile u
-            auto grad_k = [&](int u, bool half, bool first, bool last) -> bool {
+            bool due = false, prev_half = false, prev_first = false, prev_last = false;
+            // dK += dS^T Q of the tile before tile g, unless it was issued already
+            auto grad_k = [&]() -> bool {
+                if (!due) return true;
+                const int u = g - 1;
                 if (!mbar_wait(bar(DS_FULL), u & 1, abort, s.wait_limit_ns)) return false;
                 fence_after_sync();
-                mma_grad(tmem + kDK, tmem + kDP, 64, mlo + ((kSmQ + (u % QS) * kPairBytes) >> 4), mhi, id_g, half, first);
+                mma_grad(tmem + kDK, tmem + kDP, 64, mlo + ((kSmQ + (u % QS) * kPairBytes) >> 4), mhi, id_g, prev_half,
+                         prev_first);
                 mma_commit(bar(Q_EMPTY + u % QS));
-                if (last) mma_commit(bar(ACC_FULL));
+                if (prev_last) mma_commit(bar(ACC_FULL));
+                due = false;
                 return true;
             };
             for (int i = 0, item = item_at(0, ok); item < p.total_items && ok; item = item_at(++i, ok)) {
                 int bh, kb, len;
                 range(item, bh, kb, len);
-                if (len == 0) continue;
+                if (len == 0) {
+                    // the epilogue of the item before waits for this dK and reads no item until it has it, so
+                    // the ring may end before the next item that has tiles
+                    if (!(ok = grad_k())) break;
+                    continue;
+                }
                 const int T = (len + 1) / 2, kbuf = k & 1;
                 if (!(ok = mbar_wait(bar(KV_FULL + kbuf), (k >> 1) & 1, abort, s.wait_limit_ns))) break;
                 const uint32_t ka = lo + ((kSmK + kbuf * kBlockBytes) >> 4), va = lo + ((kSmV + kbuf * kBlockBytes) >> 4);
@@ -675,7 +684,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
                     fence_after_sync();
                     mma_scores(tmem + kS, ka, hi, lo + ((kSmQ + qs * kPairBytes) >> 4), hi, id_s);
                     mma_commit(bar(S_FULL));
-                    if (g >= 1 && !(ok = grad_k(g - 1, prev_half, prev_first, prev_last))) break;
+                    if (!(ok = grad_k())) break;
                     if (!(ok = mbar_wait(bar(O_FULL + os), (g / OS) & 1, abort, s.wait_limit_ns))) break;
                     fence_after_sync();
                     mma_scores(tmem + kDP, va, hi, lo + ((kSmO + os * kPairBytes) >> 4), hi, id_s);
@@ -689,11 +698,12 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
                     prev_half = half;
                     prev_first = t == 0;
                     prev_last = t == T - 1;
+                    due = true;
                 }
                 if (!ok) break;
                 ++k;
             }
-            if (ok && g > 0) ok = grad_k(g - 1, prev_half, prev_first, prev_last);
+            if (ok) ok = grad_k();
             if (!ok) record_timeout(p, 34);
             // every product this thread issued completes before TMEM is released
             int never = 0;

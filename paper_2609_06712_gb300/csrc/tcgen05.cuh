@@ -99,7 +99,9 @@ __device__ __forceinline__ bool elect_one()
 // kernels waited 2.6 % of their time for the last one at the 720p layer, 3-7 % at the
 // 12-head 480p layer (forward 900 -> 880 us, training step 4.01 -> 3.94 ms).  One producer thread fetches them ahead
 // and posts them in a ring of shared-memory slots; the other roles read them there, and a
-// slot is written again once all of them have.
+// slot is written again once all of them have.  So a role that waits inside an item keeps
+// the items kRing further on from everyone: what it waits for may depend on the item after
+// its own (the producer posts that before it works on this one) and on no later one.
 struct ItemRing {
     static constexpr int kRing = 16;
     static constexpr int kReaders = 11;      // the other producer, two more single-thread or one-warp roles, eight warps
