@@ -25,8 +25,13 @@
 //     complete, and the pipe runs dry meanwhile: one thread for all took 18.1 ms
 //     where this takes 16.0, 720p layer)
 //   key side:   S(g+1) dK(g) dP(g+1) dV(g+1) by one thread       P written over S, dS over dP
-//     (products of one thread run in order, so S(g+1) may overwrite the P(g) that
-//     dV(g) read; with S, dV and dP, dK on two threads the order drifts, and the
+//     (products are sure to run in the order they are issued in only where they share an
+//     accumulator, so S(g+1) waits until dV(g) has read its P(g), dP(g+1) until dK(g) has
+//     read its dS(g).  S and dP are a product per block of the pair, N = 64, so that the
+//     first runs while the second block's dV or dK still does.  720p training step: 54.7
+//     ms with no such wait, 58.3 waiting for whole products, 55.7 this way.
+//     With the order S dP dV dK each wait has a product in between, but P and dS have one
+//     product's time instead of two: 58.7.  With S, dV and dP, dK on two threads the
 //     kernel took 25.7 ms instead of 21.6)
 //
 // What bounds it: an M = 64, N = 128 product takes 64 cycles a K step of 16 (half
@@ -123,7 +128,7 @@ __device__ __forceinline__ void load_pair(uint32_t dst, const CUtensorMap* map, 
     }
 }
 
-// d (+)= A[smem, 64 rows, K-major] B[smem, 128 rows, K-major]^T over 128 columns
+// d = A[smem, 64 rows, K-major] B[smem, the rows of a pair or of one of its blocks, K-major]^T (id: N columns)
 __device__ __forceinline__ void mma_scores(uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t id)
 {
 #pragma unroll
@@ -132,17 +137,13 @@ __device__ __forceinline__ void mma_scores(uint32_t d, uint32_t a, uint32_t a_hi
                      kk > 0 ? 1u : 0u);
 }
 
-// d (+)= A[TMEM, 64 rows] B[smem pair, MN-major]: K steps of 16 pair rows, the second
-// block's A columns `gap` after the first's; a half tile has the first block only
-__device__ __forceinline__ void mma_grad(uint32_t d, uint32_t a, uint32_t gap, uint32_t b, uint32_t b_hi, uint32_t id,
-                                         bool half, bool first)
+// d (+)= A[TMEM, 64 rows] B[smem, one block of a pair, MN-major]: K steps of 16 of its rows
+__device__ __forceinline__ void mma_grad(uint32_t d, uint32_t a, uint32_t b, uint32_t b_hi, uint32_t id, bool first)
 {
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) mma_ts_split(d, a + kk * 8, b + kk * 128, b_hi, id, !first || kk > 0 ? 1u : 0u);
-    if (half) return;
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) mma_ts_split(d, a + gap + kk * 8, b + (kk + 4) * 128, b_hi, id, 1u);
 }
+constexpr uint32_t kSecond = (64 * 128) >> 4;     // descriptor offset from a pair's first block to its second
 
 // The 128 bytes at p into L2 (the epilogue's rows, asked for when the item starts).
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p)); }
@@ -344,8 +345,10 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dq_tc_kernel(const __g
                         if (t == 0 && k >= 1 && !(ok = mbar_wait(bar(O_EMPTY), (k - 1) & 1, abort, s.wait_limit_ns))) break;
                         if (!(ok = mbar_wait(bar(DS_FULL + db), (g >> 1) & 1, abort, s.wait_limit_ns))) break;
                         fence_after_sync();
-                        mma_grad(tmem + kDQ, tmem + kDS + db * 64, 32, mlo + ((kSmK + ks * kPairBytes) >> 4), mhi, id_g,
-                                 2 * t + 1 >= s.n_keep, t == 0);
+                        const uint32_t b = mlo + ((kSmK + ks * kPairBytes) >> 4);
+                        mma_grad(tmem + kDQ, tmem + kDS + db * 64, b, mhi, id_g, t == 0);
+                        if (2 * t + 1 < s.n_keep)           // (a half tile has the first block only)
+                            mma_grad(tmem + kDQ, tmem + kDS + db * 64 + 32, b + kSecond, mhi, id_g, false);
                         mma_commit(bar(DS_EMPTY + db));
                         mma_commit(bar(K_EMPTY + ks));
                         if (t == T - 1) mma_commit(bar(O_FULL));
@@ -463,7 +466,8 @@ constexpr uint32_t kSmO = kSmQ + QS * kPairBytes, kTiles = kSmO + OS * kPairByte
 constexpr uint32_t kS = 0, kDP = 128, kDV = 256, kDK = 384;     // TMEM columns (P over S, dS over dP)
 
 enum Bar { KV_FULL = 0, KV_EMPTY = KV_FULL + 2, Q_FULL = KV_EMPTY + 2, Q_EMPTY = Q_FULL + QS, O_FULL = Q_EMPTY + QS,
-           O_EMPTY = O_FULL + OS, S_FULL = O_EMPTY + OS, DP_FULL, P_FULL, DS_FULL, ACC_FULL, ACC_EMPTY, DRAIN, NUM_BARS };
+           O_EMPTY = O_FULL + OS, S_FULL = O_EMPTY + OS, DP_FULL, P_FULL, DS_FULL, ACC_FULL, ACC_EMPTY,
+           DV_HALF, DK_HALF, DRAIN, NUM_BARS };
 
 struct Ctrl {
     float lse2[2][128];                  // log-sum-exp (log2 units) and -D of an even / odd tile's queries
@@ -645,7 +649,7 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
     } else if (warp == kMmaWarp) {
         // ------------------------------------------------------------ S(g), dK(g - 1), dP(g), dV(g), tile by tile
         if (elect_one()) {
-            const uint32_t id_s = idesc_bf16(64, 128, false, false), id_g = idesc_bf16(64, 128, false, true);
+            const uint32_t id_s = idesc_bf16(64, 64, false, false), id_g = idesc_bf16(64, 128, false, true);
             const uint64_t dk = smem_desc(sbase, 16, 1024);          // K-major operands
             const uint64_t dm = smem_desc(sbase, 16384, 1024);       // a pair read MN-major (chunks 16 KB apart)
             const uint32_t lo = (uint32_t)dk, hi = (uint32_t)(dk >> 32), mlo = (uint32_t)dm, mhi = (uint32_t)(dm >> 32);
@@ -658,8 +662,10 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
                 const int u = g - 1;
                 if (!mbar_wait(bar(DS_FULL), u & 1, abort, s.wait_limit_ns)) return false;
                 fence_after_sync();
-                mma_grad(tmem + kDK, tmem + kDP, 64, mlo + ((kSmQ + (u % QS) * kPairBytes) >> 4), mhi, id_g, prev_half,
-                         prev_first);
+                const uint32_t b = mlo + ((kSmQ + (u % QS) * kPairBytes) >> 4);
+                mma_grad(tmem + kDK, tmem + kDP, b, mhi, id_g, prev_first);
+                mma_commit(bar(DK_HALF));
+                if (!prev_half) mma_grad(tmem + kDK, tmem + kDP + 64, b + kSecond, mhi, id_g, false);
                 mma_commit(bar(Q_EMPTY + u % QS));
                 if (prev_last) mma_commit(bar(ACC_FULL));
                 due = false;
@@ -680,20 +686,36 @@ __global__ void __launch_bounds__(kThreads, 1) sparse_bwd_dkdv_tc_kernel(const _
                 for (int t = 0; t < T; ++t, ++g) {
                     const int qs = g % QS, os = g % OS;
                     const bool half = 2 * t + 1 >= len;
+                    const uint32_t q = lo + ((kSmQ + qs * kPairBytes) >> 4), o = lo + ((kSmO + os * kPairBytes) >> 4);
                     if (!(ok = mbar_wait(bar(Q_FULL + qs), (g / QS) & 1, abort, s.wait_limit_ns))) break;
+                    // S goes where P of the tile before was, block by block once dV has read it
+                    if (g >= 1 && !(ok = mbar_wait(bar(DV_HALF), (g - 1) & 1, abort, s.wait_limit_ns))) break;
                     fence_after_sync();
-                    mma_scores(tmem + kS, ka, hi, lo + ((kSmQ + qs * kPairBytes) >> 4), hi, id_s);
+                    mma_scores(tmem + kS, ka, hi, q, hi, id_s);
+                    if (g >= 1 && !(ok = mbar_wait(bar(O_EMPTY + (g - 1) % OS), ((g - 1) / OS) & 1, abort, s.wait_limit_ns)))
+                        break;
+                    fence_after_sync();
+                    mma_scores(tmem + kS + 64, ka, hi, q + kSecond, hi, id_s);
                     mma_commit(bar(S_FULL));
                     if (!(ok = grad_k())) break;
                     if (!(ok = mbar_wait(bar(O_FULL + os), (g / OS) & 1, abort, s.wait_limit_ns))) break;
+                    // dP goes where dS of the tile before was, once dK has read it
+                    if (g >= 1 && !(ok = mbar_wait(bar(DK_HALF), (g - 1) & 1, abort, s.wait_limit_ns))) break;
                     fence_after_sync();
-                    mma_scores(tmem + kDP, va, hi, lo + ((kSmO + os * kPairBytes) >> 4), hi, id_s);
+                    mma_scores(tmem + kDP, va, hi, o, hi, id_s);
+                    if (g >= 1 && !(ok = mbar_wait(bar(Q_EMPTY + (g - 1) % QS), ((g - 1) / QS) & 1, abort, s.wait_limit_ns)))
+                        break;
+                    fence_after_sync();
+                    mma_scores(tmem + kDP + 64, va, hi, o + kSecond, hi, id_s);
                     mma_commit(bar(DP_FULL));
                     if (t == T - 1) mma_commit(bar(KV_EMPTY + kbuf));
                     if (t == 0 && k >= 1 && !(ok = mbar_wait(bar(ACC_EMPTY), (k - 1) & 1, abort, s.wait_limit_ns))) break;
                     if (!(ok = mbar_wait(bar(P_FULL), g & 1, abort, s.wait_limit_ns))) break;
                     fence_after_sync();
-                    mma_grad(tmem + kDV, tmem + kS, 64, mlo + ((kSmO + os * kPairBytes) >> 4), mhi, id_g, half, t == 0);
+                    const uint32_t om = mlo + ((kSmO + os * kPairBytes) >> 4);
+                    mma_grad(tmem + kDV, tmem + kS, om, mhi, id_g, t == 0);
+                    mma_commit(bar(DV_HALF));
+                    if (!half) mma_grad(tmem + kDV, tmem + kS + 64, om + kSecond, mhi, id_g, false);
                     mma_commit(bar(O_EMPTY + os));
                     prev_half = half;
                     prev_first = t == 0;

@@ -1,6 +1,7 @@
 """The order of waits in the persistent key-side gradient kernel, as a model: its roles (two producers, the
 log-sum-exp warp, the product issuer, the warps of the epilogue) as coroutines over counted barriers, on lists of
-work items most of which are empty.  No order of items may leave the roles waiting for one another."""
+work items most of which are empty.  No order of items may leave the roles waiting for one another, and no product
+may overwrite what one still in flight reads: products on different accumulators finish in any order."""
 import itertools
 import random
 
@@ -13,14 +14,25 @@ class Stuck(Exception):
     pass
 
 
-def run(tiles, due_across_empty=False):
-    """Runs the roles of one CTA over items of tiles[i] tiles (0: a key block no query block kept).  With
-    `due_across_empty` the issuer holds an item's last dK over the empty items after it (what must not be)."""
+class Overwritten(Exception):
+    pass
+
+
+def run(tiles, due_across_empty=False, overwrite_waits=True):
+    """Runs the roles of one CTA over items of tiles[i] tiles (0: a key block no query block kept).  What must not
+    be: with `due_across_empty` the issuer holds an item's last dK over the empty items after it, without
+    `overwrite_waits` it trusts products to finish in the order they are issued in."""
     n, done = len(tiles), {}
+    flight, order = [], random.Random(sum(tiles))       # products issued and not finished: the barriers they arrive on
     done_of = lambda name, i: done.get((name, i), 0)  # noqa: E731
 
     def arrive(name, i=0):
         done[name, i] = done_of(name, i) + 1
+
+    def product(*arrivals, over=None):     # `over`: what the product that reads its output's columns arrives on
+        if any(over in p for p in flight):
+            raise Overwritten(over)
+        flight.append(arrivals)
 
     def wait(name, i=0, count=1):          # a condition: `count` arrivals on barrier instance i
         return lambda: done_of(name, i) >= count
@@ -84,9 +96,7 @@ def run(tiles, due_across_empty=False):
             nonlocal due
             if due:
                 yield wait("ds_full", g - 1)
-                arrive("q_empty", g - 1)
-                if last:
-                    arrive("acc_full", k - 1)
+                product(("q_empty", g - 1), *([("acc_full", k - 1)] if last else []))
                 due = False
 
         for i in itertools.count():
@@ -101,18 +111,20 @@ def run(tiles, due_across_empty=False):
             k += 1
             for t in range(T):
                 yield wait("q_full", g, 2)
-                arrive("s_full", g)
+                if g and overwrite_waits:               # S goes where the last P was: dV has read it
+                    yield wait("o_empty", g - 1)
+                product(("s_full", g), over=("o_empty", g - 1))
                 k -= t == 0                             # (the tile before belongs to the item before)
                 yield from grad_k()
                 k += t == 0
+                if g and overwrite_waits:               # dP goes where the last dS was: dK has read it
+                    yield wait("q_empty", g - 1)
                 yield wait("o_full", g)
-                arrive("dp_full", g)
-                if t == T - 1:
-                    arrive("kv_empty", k - 1)
+                product(("dp_full", g), *([("kv_empty", k - 1)] if t == T - 1 else []), over=("q_empty", g - 1))
                 if t == 0 and k >= 2:
                     yield wait("acc_empty", k - 2)
                 yield wait("p_full", g)
-                arrive("o_empty", g)
+                product(("o_empty", g))
                 due, last = True, t == T - 1
                 g += 1
         yield from grad_k()
@@ -143,7 +155,10 @@ def run(tiles, due_across_empty=False):
             while w is not None and w():
                 w = waits[f] = next(roles[f], None)
                 moved = True
-        if not moved:
+        if not moved and flight:
+            for barrier in flight.pop(order.randrange(len(flight))):
+                arrive(*barrier)
+        elif not moved:
             raise Stuck([f.__name__ for f, w in waits.items() if w is not None])
 
 
@@ -168,3 +183,8 @@ def test_roles_finish_on_every_list():
 def test_model_sees_a_product_held_over_empty_items(gap):
     with pytest.raises(Stuck):
         run([1] + [0] * gap + [1], due_across_empty=True)
+
+
+def test_model_sees_a_product_that_overwrites_an_operand():
+    with pytest.raises(Overwritten):
+        run([3], overwrite_waits=False)
