@@ -352,8 +352,14 @@ __device__ __forceinline__ float fast_exp2(float x)
     return y;
 }
 
-// SiLU of a feature that enters a product in bf16: the approximate divide.
-__device__ __forceinline__ float silu(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
+// SiLU of a feature that enters a product in bf16.  The key side takes the approximate
+// divide, which is zero once 1 + e^-x passes 2^126; the query side the IEEE divide.
+struct SiluFast {
+    __device__ static float eval(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
+};
+struct SiluIeee {
+    __device__ static float eval(float x) { return x / (1.0f + __expf(-x)); }
+};
 
 // The feature maps of the activation ablation other than SiLU (Tab. abl_activation),
 // chosen at run time by `kind` (a rola_lowrank_act_t).  tanhf and erff are CUDA's
@@ -373,14 +379,22 @@ struct ActAblation {
 
 // How a bf16 kernel evaluates a pair of features.  The kernels are instantiated for the
 // default, SiLU with the rotation outside, and for any other map or placement.
+template <typename Silu>
 struct SiluOutside {
     __device__ SiluOutside(const Shape&) {}
-    __device__ float2 operator()(float u0, float u1, float2 cs) const { return rope_rotate(silu(u0), silu(u1), cs); }
+    __device__ float2 operator()(float u0, float u1, float2 cs) const
+    {
+        return rope_rotate(Silu::eval(u0), Silu::eval(u1), cs);
+    }
 };
+template <typename Silu>
 struct AnyFeature {
     int mode, kind;
     __device__ AnyFeature(const Shape& s) : mode(s.lr_rope), kind(s.lr_act) {}
-    __device__ float operator()(float x) const { return kind == ROLA_LOWRANK_ACT_SILU ? silu(x) : ActAblation{kind}(x); }
+    __device__ float operator()(float x) const
+    {
+        return kind == ROLA_LOWRANK_ACT_SILU ? Silu::eval(x) : ActAblation{kind}(x);
+    }
     __device__ float2 operator()(float u0, float u1, float2 cs) const { return lowrank_pair(u0, u1, cs, mode, *this); }
 };
 inline bool default_feature(const Shape& s)

@@ -526,8 +526,8 @@ template <int R>
 cudaError_t launch_r(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const Params& p, int ctas,
                      bool fuse, cudaStream_t st)
 {
-    return default_feature(p.s) ? launch_ra<R, SiluOutside>(mq, mk, mv, p, ctas, fuse, st)
-                                : launch_ra<R, AnyFeature>(mq, mk, mv, p, ctas, fuse, st);
+    return default_feature(p.s) ? launch_ra<R, SiluOutside<SiluFast>>(mq, mk, mv, p, ctas, fuse, st)
+                                : launch_ra<R, AnyFeature<SiluFast>>(mq, mk, mv, p, ctas, fuse, st);
 }
 
 }  // namespace

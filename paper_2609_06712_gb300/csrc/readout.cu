@@ -297,8 +297,8 @@ template <int R>
 cudaError_t launch_r(const CUtensorMap& mq, const CUtensorMap& mos, const CUtensorMap& mo, const Params& p, int ctas,
                      cudaStream_t st)
 {
-    return default_feature(p.s) ? launch_ra<R, SiluOutside>(mq, mos, mo, p, ctas, st)
-                                : launch_ra<R, AnyFeature>(mq, mos, mo, p, ctas, st);
+    return default_feature(p.s) ? launch_ra<R, SiluOutside<SiluIeee>>(mq, mos, mo, p, ctas, st)
+                                : launch_ra<R, AnyFeature<SiluIeee>>(mq, mos, mo, p, ctas, st);
 }
 
 }  // namespace
