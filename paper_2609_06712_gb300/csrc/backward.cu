@@ -803,7 +803,9 @@ __device__ __forceinline__ void mma_dfrag_x_wt(float (&acc)[R / 8][4], const flo
 
 // part[a][d] (R x 128, fp32, first r rows stored) = (+= when `add`) sum over the chunk's 64
 // tokens of A[t][a] B[t][d], A and B swizzled bf16 tiles; warp w takes the 16 x 32 output tiles
-// w, w + 4, ... (a thread adds to what it wrote itself, which is still in L2)
+// w, w + 4, ... (a thread adds to what it wrote itself, which is still in L2).  The chunk is summed
+// from zero and then added in fp32: an accumulator that starts at the sum so far loses the bits of
+// every product that lie below its own last one.
 template <int R>
 __device__ void mma_outer(uint32_t tA, uint32_t tB, int r, float* part, bool add, int warp, int lane)
 {
@@ -811,17 +813,16 @@ __device__ void mma_outer(uint32_t tA, uint32_t tB, int r, float* part, bool add
     for (int tile = warp; tile < (R / 16) * 4; tile += 4) {
         const int a0 = (tile >> 2) * 16, d0 = (tile & 3) * 32;
         float acc[4][4] = {};
+        auto at = [&](int nt, int h) {
+            return reinterpret_cast<float2*>(part + (size_t)(a0 + g + 8 * h) * kDh + d0 + 8 * nt + 2 * tig);
+        };
+        float2 old[4][2] = {};
         if (add) {
 #pragma unroll
             for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
-                    if (a0 + g + 8 * h < r) {
-                        const float2 old = *reinterpret_cast<const float2*>(part + (size_t)(a0 + g + 8 * h) * kDh + d0 +
-                                                                            8 * nt + 2 * tig);
-                        acc[nt][2 * h] = old.x;
-                        acc[nt][2 * h + 1] = old.y;
-                    }
+                    if (a0 + g + 8 * h < r) old[nt][h] = *at(nt, h);
         }
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks) {
@@ -836,12 +837,11 @@ __device__ void mma_outer(uint32_t tA, uint32_t tB, int r, float* part, bool add
             }
         }
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const int d = d0 + 8 * nt + 2 * tig;
-            if (a0 + g < r) *reinterpret_cast<float2*>(part + (size_t)(a0 + g) * kDh + d) = make_float2(acc[nt][0], acc[nt][1]);
-            if (a0 + g + 8 < r)
-                *reinterpret_cast<float2*>(part + (size_t)(a0 + g + 8) * kDh + d) = make_float2(acc[nt][2], acc[nt][3]);
-        }
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (a0 + g + 8 * h < r)
+                    *at(nt, h) = make_float2(old[nt][h].x + acc[nt][2 * h], old[nt][h].y + acc[nt][2 * h + 1]);
     }
 }
 
