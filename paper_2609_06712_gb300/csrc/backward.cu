@@ -1041,7 +1041,8 @@ __global__ void __launch_bounds__(kMT) lr_bwd_k_mma_kernel(Shape s, int group, c
     extern __shared__ __align__(128) uint8_t msm[];
     const uint32_t b0 = smem_u32(msm);
     // layout: X (k) [64] | V [64] | P [R rows] | dC [R rows]; dU takes V's place: a warp reads only its
-    // own 16 rows of V (dk~ = dC v) and writes dU to the same rows, so 48 KB at r = 32 and four CTAs an SM
+    // own 16 rows of V (dk~ = dC v) and writes dU to the same rows, so 48 KB at r = 32; the 168 registers
+    // a thread takes allow three CTAs an SM
     const uint32_t sX = b0, sV = b0 + kTile, sP = b0 + 2 * kTile, sC = sP + R * 256, sU = sV;
     const int bh = blockIdx.y, h = bh % s.H;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, tig = lane & 3;
@@ -1112,7 +1113,10 @@ __global__ void __launch_bounds__(kMT) lr_bwd_k_mma_kernel(Shape s, int group, c
 template <int R>
 size_t lr_mma_smem(bool key_side) { return (key_side ? 2 : 3) * (size_t)kTile + 2 * (size_t)R * 256; }
 
-// Chunks a CTA takes: enough CTAs for four turns of three on every SM, at most 8 chunks each.
+// Chunks a CTA takes: enough CTAs for four turns of three on each of the chip's 152 SMs (what fits up to
+// r = 32; larger ranks get more turns), at most 8 chunks each.  The count is written out, not asked of the
+// device, because the grouping is the order the partials are summed in: the same layer has the same bits
+// on a part with another number of SMs.
 int lr_group(const Shape& s)
 {
     const long long chunks = (long long)s.B * s.H * s.nC, g = chunks / (152 * 3 * 4);

@@ -167,15 +167,16 @@ struct Workspace {
     size_t prepass_slots;     // bf16 pre-pass partial slots
 };
 
-// Every kernel of the library is launched so that it may start before its predecessor
-// on the stream has drained (programmatic dependent launch): its CTAs take the space
-// that frees up and set up barriers, TMEM and descriptors; chain_begin(), which every
-// kernel executes in all CTAs before it touches global memory, then waits for the
-// predecessor's end.  Since every kernel waits, the order is transitive.  A kernel
-// releases its successor as its CTAs exit: released from the start, the successor's
-// first CTAs crowd onto the SMs that have room (an fp32 layer of 2340 tokens went from
-// 151 to 175 us, against 134 this way).  The 1024-token layer, a few microseconds a
-// kernel: 57 -> 39 us together with the RoPE table's frequencies moved to the host.
+// Every kernel of the library is launched as a programmatic dependent of its predecessor
+// on the stream.  None triggers its dependents by instruction, so a kernel's CTAs come once
+// the last CTA of the predecessor has exited; what overlaps is the launch itself, and the
+// set-up of barriers, TMEM and descriptors with the flush that ends the predecessor.
+// chain_begin(), which every kernel executes in all CTAs before it touches global memory,
+// waits for that end.  Since every kernel waits, the order is transitive.  (A trigger at the
+// start of every kernel lets the successor's first CTAs crowd onto the SMs that have room:
+// an fp32 layer of 2340 tokens went from 151 to 175 us, against 134 this way.)  The
+// 1024-token layer, a few microseconds a kernel: 57 -> 39 us together with the RoPE
+// table's frequencies moved to the host (35 now, the fp32 layer 131).
 template <typename... P, typename... A>
 cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args)
 {
@@ -405,14 +406,5 @@ inline bool default_feature(const Shape& s)
 // Byte offset of 16-byte chunk c of row r in a [rows][128 bf16] tile with the
 // chunk index XOR-swizzled by the row (conflict-free ldmatrix on 8-row groups).
 __device__ __forceinline__ uint32_t sw128(int r, int c) { return r * 256 + ((c ^ (r & 7)) << 4); }
-
-// Byte offset of 16-byte chunk c (0..15) of row r in a 64-row block tile as a
-// [chunk][row][64] TMA box with 128-byte swizzle writes it: the two 64-wide
-// halves of a row are 8 KB apart, and within 1024-byte atoms chunk c & 7 of
-// row r sits at (c & 7) ^ (r & 7).
-__device__ __forceinline__ uint32_t tsw(int r, int c)
-{
-    return (c >> 3) * 8192 + r * 128 + (((c & 7) ^ (r & 7)) << 4);
-}
 
 }  // namespace rola

@@ -18,7 +18,7 @@
 // (k, v and q boxes of 32 x 128, 8 KB each), which keeps a CTA small enough
 // that two fit on an SM for r <= 64 (16 warps per SM hide the latency of the
 // dependent MMA and rotation chains; r = 64 with one CTA an SM took 914 us for the
-// summary of 40 heads and 75600 tokens, 562 with two).  Per half, 8 warps:
+// summary of 40 heads and 75600 tokens, 562 with two and 526 now).  Per half, 8 warps:
 //   rotate q, k (warp w = token rows 4w .. 4w + 3, lane = 4 coordinates),
 //   store q^r, k^r, pool; U = K P_k^T (mma.sync; warp = 16 tokens x a quarter
 //   or half of the r columns); k~ = R_r SiLU(U) to shared memory; the half's

@@ -16,9 +16,10 @@
 // two O^s buffers (one for r > 64), filled by its own TMA loads, so the warps of an
 // SM are at different points of the chain and their loads, products and stores
 // overlap.  Bound by HBM: 768 B per (head, token).  720p layer (40 heads, 75600
-// tokens): r = 32 496 -> 440 us (5.3 TB/s), r = 64 1048 -> 624 us; the form before
+// tokens): r = 32 496 -> 350 us (6.6 TB/s), r = 64 1048 -> 552 us; the form before
 // (64-token units over 8 warps with three CTA barriers each, one or two CTAs an SM)
-// waited on its own chain most of the time.
+// waited on its own chain most of the time.  From r = 64 the features' IEEE divides
+// weigh (an approximate one, which loses features below -87: 464 us).
 #include <cudaTypedefs.h>
 
 #include "common.cuh"

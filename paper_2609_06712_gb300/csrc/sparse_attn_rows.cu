@@ -63,12 +63,13 @@
 //   - two softmax groups in turn: 11.85 -> 11.5 ms (QN = 64), 8.2 -> 7.3 ms (QN = 128).
 //   - cube blocks on this kernel instead of a transposed form of their own: 4.88 ->
 //     3.43 ms (40 heads, 21 x 30 x 52 grid, 62 of 624 cubes kept).
-//   - items off a counter instead of dealt out evenly: 11.5 -> 11.2 ms (QN = 64).
+//   - items off a counter instead of dealt out evenly: 11.5 -> 11.1 ms (QN = 64).
 //   - QN = 64 takes ~1240 cycles a tile: 1024 of tensor work (an M = 64 product
 //     runs at half the M = 128 rate) and 144 KB through the shared memory (1125 at
 //     128 B/cycle).  QN = 128 takes ~1350 against the same 1024.  The 1400 W power
 //     cap sets the clock: 1.95-2.03 GHz for QN = 64, 1.72-1.82 GHz for QN = 128,
-//     whose 1650 TFLOP/s are 0.95 of the rate a GEMM sustains under that cap.
+//     whose 1650-1700 TFLOP/s (7.1-6.9 ms, by the clock) are 0.95-0.98 of the rate a
+//     GEMM sustains under that cap.
 //
 // Per 64-query block and 128-key tile the shared memory sees 64 KB of TMA
 // writes (K, V) and 80 KB of operand reads (Q 16, K 32, V 32) for 4.2 MFLOP,

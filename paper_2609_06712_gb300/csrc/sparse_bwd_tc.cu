@@ -34,16 +34,16 @@
 //     product's time instead of two: 58.7.  With S, dV and dP, dK on two threads the
 //     kernel took 25.7 ms instead of 21.6)
 //
-// What bounds it: an M = 64, N = 128 product takes 64 cycles a K step of 16 (half
-// the M = 128 rate), 1536 (query side) and 2048 (key side) tensor cycles a
-// tile; shared memory moves 192 / 224 KB a tile (1500 / 1750 cycles at 128
+// What bounds it: an M = 64 product takes 64 cycles a K step of 16 with N = 128 (half
+// the M = 128 rate) and 45 with N = 64, so 1536 (query side) and 2464 (key side) tensor
+// cycles a tile; shared memory moves 192 / 256 KB a tile (1500 / 2000 cycles at 128
 // B/cycle).  The transposed form used before (M = 128 x N = 64 products, 1152
 // and 1536 tensor cycles, P and dS through shared memory) moved 224 and 288 KB,
 // and its two-deep rings of 64 KB pairs were held through the whole tile.  At
 // the 720p layer (40 heads, 75600 tokens, 118 of 1182 blocks kept): query side
-// 27.3 -> 16.0 ms, key side 37.9 -> 21.9 ms (872 / 1192 ns a tile; the products
-// alone take 750 / 1000 ns at the 2.05 GHz the SMs hold under this load); at
-// the 12-head 480p layer 1.84 -> 0.99 and 2.52 -> 1.40 ms.
+// 27.3 -> 15.9 ms, key side 37.9 -> 22.5 ms (866 / 1226 ns a tile; the products
+// alone take 750 / 1200 ns at the 2.05 GHz the SMs hold under this load); at
+// the 12-head 480p layer 1.84 -> 0.99 and 2.52 -> 1.41 ms.
 //
 // Roles (384 threads, one persistent CTA per SM):
 //   warps 0-7  P / dS and the epilogue; warp w owns TMEM lane quarter w mod 4
